@@ -56,7 +56,9 @@ typedef enum {
 } fv_status;
 
 typedef enum {
-  FV_VANILLA = 0,   /* full T x K uint16 backpointer table + backtrack (Sec. III-A) */
+  FV_VANILLA = 0,   /* full table + backtrack (Sec. III-A): T x K uint16 backpointers,
+                       or T x K delta values (128 < K <= 1024, where the workspace
+                       has room: fv_workspace_size asks for them)               */
   FV_FLASH = 1,     /* non-recursive D&C with MidState (Alg. 1, Alg. 2)            */
   FV_BEAM = 2,      /* dynamic beam (Sec. V-C); P >= 1 makes it FLASH-BS          */
   FV_CHECKPOINT = 3 /* Checkpoint Viterbi, the baseline of Sec. II-A (see below)  */
@@ -275,7 +277,7 @@ int32_t fv_set_engine_variant(int32_t K, int32_t variant);
  * the scratch lives in a file-scope device array of
  * FV_NOALLOC_SCRATCH_BYTES (16 MiB) that every GPU loading the library holds
  * until the process exits.  batch->T_host is required; a request whose
- * workspace (fv_workspace_size for FV_VANILLA) exceeds that size is rejected
+ * workspace with uint16 backpointers exceeds that size is rejected
  * with FV_ENOMEM before anything is enqueued.  No cudaMalloc, cudaFree or
  * other allocating routine is called.
  *

@@ -237,6 +237,8 @@ struct Layout {
   size_t ap, snapx;  // streamed exact configurations (K > 256)
   size_t wide;       // whole-GPU configuration scratch (K > 1024)
   size_t at;         // column-major logA copy of the streamed configurations (256 < K <= 1024)
+  size_t prune;      // bounded-row engine: copies and column lists of the largest model, then
+  size_t guess, guess_bytes;  // the trace's segment ends
   uint64_t aux_elems;
   int64_t map_stride, snap_stride, list_cap;
   int32_t Wcap, Bcap, pe_cap, max_ctas;
@@ -249,13 +251,22 @@ int32_t beam_wcap(const fv_model* models, int32_t n_models, int32_t B) {
   return std::min(std::max(B, 1), kmax);
 }
 
+// Exact decoding keeps delta rows (T x K floats) instead of psi rows when
+// every model of the batch runs the bounded-row engine.
+bool delta_rows(const fv_model* models, int32_t n_models, int mode) {
+  if (mode != FV_VANILLA) return false;
+  for (int m = 0; m < n_models; ++m)
+    if (models[m].trans != FV_TRANS_DENSE || !dense_prune_K(models[m].K)) return false;
+  return true;
+}
+
 // Workspace layout of a request.  fp: task-level plan (FLASH, and BEAM
 // with P >= 1).  The per-sequence aux area holds: vanilla, T*K uint16
 // backpointers; flash and FLASH-BS, T floats of delta along the path; beam
 // with P = 0, T*Wcap int32 state ids (a second area of the same size holds
 // the source slots).
 Layout layout_for(const fv_model* models, int32_t n_models, const fv_batch* b, int mode, const FlashPlan* fp,
-                  int32_t B = 0, int32_t ckpt_P = 0) {
+                  int32_t B = 0, int32_t ckpt_P = 0, bool rows32 = false) {
   Layout L;
   memset(&L, 0, sizeof(L));
   const int32_t n = b->n_seq;
@@ -269,7 +280,9 @@ Layout layout_for(const fv_model* models, int32_t n_models, const fv_batch* b, i
   L.qlast = align_up(L.order + sizeof(int32_t) * (size_t)n);
   L.aux = align_up(L.qlast + sizeof(int32_t) * (size_t)n);
   uint64_t aux = 0;
+  int64_t sum_T = 0;
   for (int i = 0; i < n && b->T_host; ++i) {
+    sum_T += b->T_host[i];
     const int m = b->model_host ? b->model_host[i] : 0;
     const uint64_t T = (uint64_t)b->T_host[i], K = (uint64_t)models[m].K;
     if (mode == FV_VANILLA) aux += (T * K + 7ull) & ~7ull;
@@ -278,7 +291,16 @@ Layout layout_for(const fv_model* models, int32_t n_models, const fv_batch* b, i
     else aux += (T + 3ull) & ~3ull;
   }
   L.aux_elems = aux;
-  size_t end = align_up(L.aux + aux * (mode == FV_VANILLA ? 2 : 4));
+  size_t end = align_up(L.aux + aux * (mode == FV_VANILLA && !rows32 ? 2 : 4));
+  if (rows32) {
+    size_t area = 0;
+    for (int m = 0; m < n_models; ++m) area = std::max(area, prune_area_bytes(models[m].K));
+    L.prune = end;
+    L.guess = align_up(area);  // from L.prune
+    L.guess_bytes = prune_guess_bytes(aux, n, sum_T);
+    L.total = align_up(end + L.guess + L.guess_bytes);
+    return L;
+  }
   if (beam0) {
     L.aux2 = end;
     end = align_up(L.aux2 + 4 * (size_t)aux);
@@ -606,8 +628,19 @@ size_t fv_workspace_size(const fv_model* models, int32_t n_models, const fv_batc
   }
   if (p->mode == FV_BEAM && p->B < 1) return 0;
   if (p->mode != FV_VANILLA && p->mode != FV_BEAM && p->mode != FV_CHECKPOINT) return 0;
-  return layout_for(models, n_models, batch, p->mode, nullptr, p->B, p->P).total;
+  const size_t base = layout_for(models, n_models, batch, p->mode, nullptr, p->B, p->P).total;
+  if (!delta_rows(models, n_models, p->mode)) return base;
+  return std::max(base, layout_for(models, n_models, batch, p->mode, nullptr, 0, 0, true).total);
 }
+
+}  // extern "C"
+
+size_t fv::exact_min_workspace(const fv_model* models, int32_t n_models, const fv_batch* batch) {
+  if (!batch || !batch->T_host || check_common(models, n_models, batch) != FV_OK) return 0;
+  return layout_for(models, n_models, batch, FV_VANILLA, nullptr).total;
+}
+
+extern "C" {
 
 fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* batch, const fv_params* p_in,
                     void* workspace, size_t ws_bytes, int32_t* paths_out, float* scores_out,
@@ -636,10 +669,26 @@ fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* ba
   if (tasks)
     fp = plan_flash(models, n_models, batch, p->P, p->mode == FV_FLASH ? p->mem_budget_bytes : 0,
                     (p->flags & FV_NO_SORT) != 0);
-  const Layout L = layout_for(models, n_models, batch, p->mode, tasks ? &fp : nullptr, p->B, p->P);
+  Layout L = layout_for(models, n_models, batch, p->mode, tasks ? &fp : nullptr, p->B, p->P);
+  // exact decoding by the bounded-row engine, where the workspace holds the
+  // delta rows (a workspace of the smaller, psi-row size keeps the others)
+  bool prune = batch->T_host && n > 0 && delta_rows(models, n_models, p->mode);
+  for (int m = 0; m < n_models && prune; ++m)
+    prune = dense_uses_prune(models[m].K, (p->flags & FV_NO_TUNE) != 0, (p->flags & FV_TEST_WITHHOLD_STEP) != 0);
+  if (prune) {
+    const Layout LP = layout_for(models, n_models, batch, p->mode, nullptr, 0, 0, true);
+    prune = ws_bytes >= LP.total;
+    if (prune) {
+      // the copies go to the end of the workspace: whatever lies between is
+      // room for the rows
+      const size_t area = LP.total - LP.prune;
+      L = LP;
+      L.prune = (ws_bytes - area) & ~(kAlign - 1);
+    }
+  }
   if (batch->T_host && ws_bytes < L.total) return FV_ENOMEM;
   if (ws_bytes < L.aux) return FV_ENOMEM;
-  const uint64_t cap = (ws_bytes - L.aux) / (p->mode == FV_VANILLA ? 2 : 4);
+  const uint64_t cap = prune ? (L.prune - L.aux) / 4 : (ws_bytes - L.aux) / (p->mode == FV_VANILLA ? 2 : 4);
   if (n == 0) return FV_OK;
 
   char* ws = static_cast<char*>(workspace);
@@ -701,6 +750,26 @@ fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* ba
     da.wide_withhold = (p->flags & FV_TEST_WITHHOLD_STEP) ? 1 : 0;
     da.no_tune = (p->flags & FV_NO_TUNE) ? 1 : 0;
     da.hdr = hdr;
+    if (prune) {
+      da.kind = kJobVanilla;
+      da.pr_D = reinterpret_cast<float*>(ws + L.aux);
+      if (launch_prune_prep(md.logA, md.K, ws + L.prune, &da, st) != cudaSuccess) return FV_ECUDA;
+      int64_t sum_T = 0, all_T = 0;
+      int32_t max_T = 1;
+      for (int i = 0; i < n; ++i) {
+        all_T += batch->T_host[i];
+        if ((batch->model_host ? batch->model_host[i] : 0) != m) continue;
+        sum_T += batch->T_host[i];
+        max_T = std::max(max_T, batch->T_host[i]);
+      }
+      timed_begin(st);
+      if (launch_prune_forward(da, sum_T, max_T, st) != cudaSuccess) return FV_ECUDA;
+      timed_end(st);
+      if (launch_prune_trace(da, reinterpret_cast<int32_t*>(ws + L.prune + L.guess), L.guess_bytes, all_T, max_T,
+                             paths_out, st) != cudaSuccess)
+        return FV_ECUDA;
+      continue;
+    }
     {
       int kpm = 0, cols = 0;
       dense_stream_geometry(md.K, &kpm, &cols);

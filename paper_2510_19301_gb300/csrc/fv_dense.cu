@@ -1447,6 +1447,11 @@ void dense_set_variant(int K, int v) {
 }
 int dense_get_variant(int K) { return g_variant[dense_k_class(K)]; }
 
+bool dense_prune_K(int K) { return K > 128 && K <= 1024; }
+bool dense_uses_prune(int K, bool no_tune, bool withhold) {
+  return dense_prune_K(K) && !withhold && (no_tune || g_variant[dense_k_class(K)] == 0);
+}
+
 cudaError_t launch_dense_forward(DenseArgs a, int max_clusters, cudaStream_t st) {
   if (a.K > 1024) return launch_wide_forward(a, st);
   const int v = a.no_tune ? 0 : g_variant[dense_k_class(a.K)];

@@ -126,6 +126,13 @@ struct DenseArgs {
                               // (streamed and whole-GPU configurations: the exact re-scan reads it)
   int32_t wide_withhold;      // test hook: CTA 0 of the whole-GPU engine never publishes its step count;
                               // CTA 1 of each 4- / 8-CTA cluster withholds its second-tick arrivals
+  // bounded-row engine (fv_prune.cu; null: not prepared): padded row copy of
+  // logA, per column the list of its largest weights, their rows, the cutoff
+  const float* pr_A;
+  const float* pr_val;
+  const uint16_t* pr_row;
+  const float* pr_cut;
+  float* pr_D;                // delta rows, T x K floats per sequence at job.aux_off
   int32_t no_tune;            // use the default engine configuration, not the tuned one
   WsHeader* hdr;
 };
@@ -207,6 +214,10 @@ struct ScoreArgs {
   const int32_t* obs;
 };
 
+// Smallest workspace that exact decoding of dense models runs in (psi rows;
+// fv_workspace_size asks for delta rows where the bounded-row engine decodes).
+size_t exact_min_workspace(const fv_model* models, int32_t n_models, const fv_batch* batch);
+
 int dense_supported_K(int K);
 // Engine configuration variants of a K class and the tuned choice.
 int dense_k_class(int K);
@@ -221,6 +232,17 @@ cudaError_t launch_wide_forward(DenseArgs a, cudaStream_t st);
 // small state spaces (K <= 128), every job kind: a CTA of K-class threads per
 // job, a thread per state (fv_small.cu)
 cudaError_t launch_small_forward(const DenseArgs& a, cudaStream_t st);
+// bounded-row engine (fv_prune.cu), exact decoding at 128 < K <= 1024: bytes
+// of a model's copies and column lists, their preparation, the forward
+// launch (delta rows to a.pr_D) and the backtrack from those rows
+size_t prune_area_bytes(int K);
+cudaError_t launch_prune_prep(const float* logA, int K, char* area, DenseArgs* a, cudaStream_t st);
+cudaError_t launch_prune_forward(const DenseArgs& a, int64_t sum_T, int max_T, cudaStream_t st);
+size_t prune_guess_bytes(uint64_t aux_elems, int32_t n_seq, int64_t sum_T);
+cudaError_t launch_prune_trace(const DenseArgs& a, int32_t* guess, size_t guess_bytes, int64_t sum_T, int max_T,
+                               int32_t* paths, cudaStream_t st);
+bool dense_prune_K(int K);
+bool dense_uses_prune(int K, bool no_tune, bool withhold);
 // AT[j * KD + i] = logA[i * K + j] (rows K..KD-1 are -inf), KD = wide_lane_stride(K).
 cudaError_t launch_wide_transpose(const float* logA, int K, float* AT, cudaStream_t st);
 void dense_stream_geometry(int K, int* KPM, int* cols);

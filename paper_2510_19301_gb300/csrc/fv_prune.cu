@@ -1,0 +1,889 @@
+// fv_prune.cu -- the exact forward engine with bounded candidate rows (exact
+// decoding, dense transitions, 128 < K <= 1024).
+//
+// The max-plus step (Sec. III-A) needs, for every target j, the maximum over
+// i of fl(delta[i] + A[i][j]).  Evaluating all K rows is bound by the FP32
+// max (64 candidates per clock per SM), and most rows cannot win.  Here a
+// column keeps the list of its M largest weights and a cutoff b_j, the
+// largest weight outside the list.  A row i outside the list of j gives at
+// most fl(delta[i] + b_j) (rounding is monotone), so once a target holds a
+// candidate above that it needs no row with a smaller delta.  Per step a warp
+//   1. forms the M listed candidates of its targets, and the candidates of
+//      the rows with delta >= max(delta) - gap (its gap follows what its last
+//      steps needed);
+//   2. from the best candidates so far computes the smallest delta that could
+//      still reach a target, and forms the candidates of the rows between
+//      that and the first threshold.
+// Only the maximum is kept: delta_t = fl(max + E_t) is exact on any input (an
+// input that bounds badly only runs more rows), delta rows go to the
+// workspace, and the backtrack recomputes the argmax of the path's own states
+// (below), K candidates per step instead of K^2 backpointers.  On Dirichlet(1)
+// weights with log-softmax normal emissions a step takes about 34 of 256 rows,
+// 40 of 512, 61 of 1000.
+//
+// Measured (GB300): 1024 sequences of 500 .. 4000 steps, K = 256: 17.4 -> 7.7
+// ms per decode against the slot engine of fv_dense.cu; 150 sequences of 200
+// .. 1500 steps, K = 1000: 21.8 -> 8.7 ms; one K = 512 sequence of 512 steps:
+// 1.81 -> 1.34 ms.  Bound now: latency and shared-memory wavefronts (at K =
+// 256, 650 wavefronts and 2200 warp instructions per job step), not the max.
+#include <cuda_runtime.h>
+#include <float.h>
+#include <math_constants.h>
+#include <stdint.h>
+
+#include "fv_internal.cuh"
+#include "fv_launch.h"
+
+namespace fv {
+
+// ------------------------------------------------------------------- prep
+// Order-preserving key of a float (larger float, larger key); 0 is below
+// every key of a number.
+__device__ __forceinline__ uint32_t ord_key(float x) {
+  const uint32_t u = __float_as_uint(x);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+__device__ __forceinline__ float ord_value(uint32_t k) {
+  return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
+}
+
+// Padded row copy of logA (stride KP, columns beyond K -inf) and, per
+// column, the cutoff and the list of the rows above it, in ascending row
+// order: the largest cutoff with at most M rows above it, found by bisecting
+// the keys (a warp per column, VPL keys per lane in registers).
+// One CTA takes 8 adjacent columns, staged column-major in shared memory so
+// that global loads read whole 32-byte sectors.
+template <int VPL>
+__global__ void __launch_bounds__(256) prune_prep_kernel(const float* logA, int K, int KP, int M, float* Apad,
+                                                         float* lval, uint16_t* lrow, float* cut) {
+  extern __shared__ float scol[];  // [8][32 * VPL + 4]
+  constexpr int ST = 32 * VPL + 4;
+  const int j0 = blockIdx.x * 8, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  for (int x = tid; x < 8 * K; x += 256) {
+    const int i = x >> 3, c = x & 7;
+    const float v = j0 + c < K ? __ldg(logA + (int64_t)i * K + j0 + c) : -CUDART_INF_F;
+    scol[c * ST + i] = v;
+    Apad[(int64_t)i * KP + j0 + c] = v;
+  }
+  __syncthreads();
+  const int j = j0 + warp;
+  uint32_t key[VPL];
+#pragma unroll
+  for (int k = 0; k < VPL; ++k) {
+    const int i = 32 * k + lane;
+    key[k] = (i < K && j < K) ? ord_key(scol[warp * ST + i]) : 0u;
+  }
+  uint32_t prefix = 0, lim = 0;  // the list: keys >= lim (lim 0: keys > prefix)
+  for (int bit = 31; bit >= 0; --bit) {
+    const uint32_t tr = prefix | (1u << bit);
+    int c = 0;
+#pragma unroll
+    for (int k = 0; k < VPL; ++k) c += key[k] >= tr;
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (c == M) {
+      lim = tr;
+      break;
+    }
+    if (c > M) prefix = tr;
+  }
+  if (!lim) lim = prefix + 1;
+  uint32_t top = 0;
+  int base = 0;
+#pragma unroll
+  for (int k = 0; k < VPL; ++k) {
+    const bool in = key[k] >= lim && key[k] != 0u;
+    if (!in && key[k] > top) top = key[k];
+    const uint32_t m = __ballot_sync(0xffffffffu, in);
+    const int p = base + __popc(m & ((1u << lane) - 1u));
+    if (in && p < M) {
+      lval[(int64_t)p * KP + j] = ord_value(key[k]);
+      lrow[(int64_t)p * KP + j] = (uint16_t)(32 * k + lane);
+    }
+    base += __popc(m);
+  }
+  top = __reduce_max_sync(0xffffffffu, top);
+  for (int p = base + lane; p < M; p += 32) {
+    lval[(int64_t)p * KP + j] = -CUDART_INF_F;
+    lrow[(int64_t)p * KP + j] = 0;
+  }
+  if (lane == 0) cut[j] = top ? ord_value(top) : -CUDART_INF_F;
+}
+
+// ----------------------------------------------------------------- engine
+// (NaN operands are passed over)
+__device__ __forceinline__ float warp_max_f32(float x) {
+  float r;
+  asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float warp_min_f32(float x) {
+  float r;
+  asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
+// A delta below the result gives fl(delta + b) < best: the margin of 2^-22
+// of the magnitudes covers the roundings of the difference, of the margin
+// and of the sum.  best = -inf gives -inf (every finite delta matters).
+__device__ __forceinline__ float need_delta(float best, float b) {
+  return __fmaf_rn(-2.384185791e-7f, __fadd_rn(fabsf(best), fabsf(b)), __fadd_rn(best, -b));
+}
+__device__ __forceinline__ float ld_stream(const float* p) {
+  float v;
+  asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+template <int C>
+__device__ __forceinline__ void ld_stream_vec(const float* p, float (&e)[C]) {
+  if constexpr (C == 4)
+    asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(e[0]), "=f"(e[1]), "=f"(e[2]), "=f"(e[3])
+                 : "l"(p));
+  else if constexpr (C == 2)
+    asm volatile("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(e[0]), "=f"(e[1]) : "l"(p));
+}
+// C adjacent weights of one row
+template <int C>
+struct Vec {
+  float v[C];
+  __device__ __forceinline__ void lds(const float* p) {
+    if constexpr (C == 4) {
+      const float4 x = *reinterpret_cast<const float4*>(p);
+      v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    } else if constexpr (C == 2) {
+      const float2 x = *reinterpret_cast<const float2*>(p);
+      v[0] = x.x; v[1] = x.y;
+    } else {
+      v[0] = *p;
+    }
+  }
+  __device__ __forceinline__ void ldg(const float* p) {
+    if constexpr (C == 4) {
+      const float4 x = __ldg(reinterpret_cast<const float4*>(p));
+      v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    } else if constexpr (C == 2) {
+      const float2 x = __ldg(reinterpret_cast<const float2*>(p));
+      v[0] = x.x; v[1] = x.y;
+    } else {
+      v[0] = __ldg(p);
+    }
+  }
+};
+
+constexpr int kPruneAhead = 3;  // emission scores loaded this many steps ahead
+// KP = padded state count, CL = CTAs (a cluster) that split a job's columns,
+// C = adjacent columns per lane (a job takes W = KP / (32 CL C) warps of each
+// CTA), G = jobs side by side, RES = the CTA's columns of logA are resident
+// in shared memory (else rows are read through L1 / L2), M = column list
+// length.
+template <int KP, int CL, int C, int G, bool RES, int M>
+struct PruneCfg {
+  static constexpr int KH = KP / CL, W = KH / (32 * C), NT = G * W * 32, NW = KP / 32;
+  static constexpr int WB = NW < 8 ? NW : 8;  // words (of 32 rows) per list batch
+  static constexpr int U = RES ? 4 : 8;       // rows in flight (shared memory / L2 latency)
+  // row list entries of a warp (a batch may add 32 WB to a list that is not yet full)
+  static constexpr int CAP = (NW <= WB ? KP : 32 * WB + 128) + 2 * U;
+  static constexpr size_t a_bytes = RES ? (size_t)KP * KH * 4 : 0;
+  static constexpr size_t d_bytes = (size_t)G * 2 * KP * 4;  // delta, double buffered
+  static constexpr size_t l_bytes = (size_t)G * W * CAP * 8;
+  static constexpr size_t smem = a_bytes + d_bytes + l_bytes;
+};
+// bounded wait of the cluster exchange (~1 s at 2 GHz)
+constexpr long long kPruneWaitCycles = 1ll << 31;
+
+template <int KP, int CL, int C, int G, bool RES, int M>
+__global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_fwd_kernel(DenseArgs a) {
+  using Cfg = PruneCfg<KP, CL, C, G, RES, M>;
+  constexpr int KH = Cfg::KH, W = Cfg::W, NT = Cfg::NT, NW = Cfg::NW, CAP = Cfg::CAP, WB = Cfg::WB, U = Cfg::U;
+  extern __shared__ __align__(16) char smem[];
+  __shared__ __align__(8) uint64_t s_bar[G][2];
+  __shared__ int s_abort;
+  __shared__ uint32_t s_stop[CL];
+  const bool stop = a.hdr->status != 0;  // an earlier kernel recorded an error
+  if (CL == 1 && stop) return;
+  const int K = a.K;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int grp = warp / W, gw = warp % W, gt = gw * 32 + lane;  // job group, its warp and thread
+  const uint32_t rank = CL > 1 ? cluster_ctarank() : 0u;
+  const int col0 = (int)rank * KH + gt * C;
+  const uint32_t lt = (1u << lane) - 1u;
+  char* sA = smem + gt * C * 4;
+  float* sd = reinterpret_cast<float*>(smem + Cfg::a_bytes) + grp * 2 * KP;
+  float2* list = reinterpret_cast<float2*>(smem + Cfg::a_bytes + Cfg::d_bytes) + warp * CAP;
+  // barrier of the job's warps here; true where any thread passes true
+  auto group_any = [&](bool x) -> bool {
+    if constexpr (W == 1) {
+      return __any_sync(0xffffffffu, x);
+    } else {
+      uint32_t r;
+      asm volatile(
+          "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, %2, %3, p;\n\t"
+          "selp.u32 %0, 1, 0, q;\n\t}"
+          : "=r"(r)
+          : "r"((uint32_t)x), "r"(grp + 1), "n"(W * 32)
+          : "memory");
+      return r != 0;
+    }
+  };
+  if constexpr (RES) {
+    const float4* src = reinterpret_cast<const float4*>(a.pr_A);
+    float4* dst = reinterpret_cast<float4*>(smem);
+    for (int x = threadIdx.x; x < K * (KH / 4); x += NT)
+      dst[x] = __ldg(src + (x / (KH / 4)) * (KP / 4) + rank * (KH / 4) + x % (KH / 4));
+  }
+  const char* __restrict__ gA = reinterpret_cast<const char*>(a.pr_A + col0);
+  constexpr int RB = (RES ? KH : KP) * 4;  // bytes of a row of the copy that is read
+  // the columns' lists stay in registers: values, row offsets (4 * row)
+  float lv[M][C], cut[C];
+  uint32_t lr[M][(C + 1) / 2];
+#pragma unroll
+  for (int x = 0; x < M; ++x)
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      lv[x][c] = __ldg(a.pr_val + x * KP + col0 + c);
+      const uint32_t r = 4u * __ldg(a.pr_row + x * KP + col0 + c);
+      lr[x][c / 2] = c % 2 ? (lr[x][c / 2] | (r << 16)) : r;
+    }
+#pragma unroll
+  for (int c = 0; c < C; ++c) cut[c] = __ldg(a.pr_cut + col0 + c);
+  uint32_t peer[CL];  // the other CTAs' shared memory
+  const uint32_t self = smem_addr(smem);
+  if (threadIdx.x == 0) s_abort = 0;
+  if constexpr (CL > 1) {
+#pragma unroll
+    for (int r = 0; r < CL; ++r) peer[r] = dsmem_addr(smem, r);
+    if (threadIdx.x < 2 * G) {
+      mbar_init(smem_addr(&s_bar[0][0] + threadIdx.x), 1);
+      fence_mbar_init_cluster();
+    }
+    cluster_sync_all();  // every CTA of the cluster runs and its barriers are ready
+    // the decision to stop is the cluster's: every CTA sees every flag
+    if (threadIdx.x < CL) dsmem_st_u32(dsmem_addr(&s_stop[rank], threadIdx.x), stop ? 1u : 0u);
+    cluster_sync_all();
+    bool any = false;
+#pragma unroll
+    for (int r = 0; r < CL; ++r) any |= s_stop[r] != 0;
+    if (any) return;
+  } else {
+    __syncthreads();
+  }
+  const int count = a.order_count;
+  // job slots of the launch; a slot's jobs: longest first, rows of slots
+  // forwards and backwards in turn, so every SM gets about the same steps
+  // (every CTA of a cluster computes the same job without a message)
+  const int ncl = (int)gridDim.x / CL, slots = ncl * G;
+  const int cid = (int)blockIdx.x / CL;
+  const int slot = grp * ncl + ((grp & 1) ? ncl - 1 - cid : cid);
+  bool live = true;
+  uint32_t ph = 0;  // steps run so far: buffer ph & 1, its (ph >> 1)-th use
+
+  for (int round = 0;; ++round) {
+    const int job = round * slots + ((round & 1) ? slots - 1 - slot : slot);
+    if (round * slots >= count) break;
+    if (job >= count) continue;
+    const int b = a.order[a.order_begin + job];
+    const Job jb = a.jobs[b];
+    const int T = jb.T;
+    const bool dense = a.emit == FV_EMIT_DENSE;
+    // emission scores of the next kPruneAhead steps, oldest first; symbols
+    // are read one step before the table entries they select
+    float er[kPruneAhead][C];
+    int xs = 0;
+    const float* ep = dense ? a.E + jb.e_off + col0 : nullptr;  // row of the next load
+    float* dt = a.pr_D + jb.aux_off + col0;                     // row of this step's delta
+    const bool vec = dense && C > 1 && K % C == 0 && ((reinterpret_cast<uintptr_t>(ep) & (4 * C - 1)) == 0);
+    auto load_e = [&](int t, float (&e)[C]) {
+      if (vec) {
+        // whole pieces of an aligned row
+        if (t < T && col0 < K) ld_stream_vec<C>(ep, e);
+        ep += K;
+        return;
+      }
+      if (dense) {
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+          if (t < T && col0 + c < K) e[c] = ld_stream(ep + c);
+        ep += K;
+        return;
+      }
+#pragma unroll
+      for (int c = 0; c < C; ++c)
+        if (t < T && col0 + c < K) e[c] = __ldg(a.logB + (int64_t)(col0 + c) * a.V + xs);
+      if (t + 1 < T) xs = __ldg(a.obs + jb.e_off + t + 1);
+    };
+    if (!dense) xs = __ldg(a.obs + jb.e_off);
+#pragma unroll
+    for (int k = 0; k < kPruneAhead; ++k) {
+#pragma unroll
+      for (int c = 0; c < C; ++c) er[k][c] = 0.f;
+      load_e(k, er[k]);
+    }
+    float gap = 0.f;  // how far below the maximum this warp's last steps had to look
+    for (int t = 0; t < T; ++t, ++ph) {
+      const uint32_t cur = ph & 1u;  // buffer written by this step; cur ^ 1 is read
+      float e[C];
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        e[c] = er[0][c];
+#pragma unroll
+        for (int k = 0; k + 1 < kPruneAhead; ++k) er[k][c] = er[k + 1][c];
+      }
+      load_e(t + kPruneAhead, er[kPruneAhead - 1]);
+      float dval[C];
+      const float* dl = sd + (cur ^ 1u) * KP;
+      if (t == 0) {
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+          dval[c] = col0 + c < K ? __fadd_rn(__ldg(a.log_pi + col0 + c), e[c]) : -CUDART_INF_F;
+      } else {
+        constexpr bool KEEP = NW <= 8;  // the deltas of this lane stay in registers
+        float dk[WB], dmax = -CUDART_INF_F;
+#pragma unroll
+        for (int k = 0; k < NW; ++k) {
+          const float d = dl[32 * k + lane];
+          if constexpr (KEEP) dk[k] = d;
+          dmax = fmaxf(dmax, d);
+        }
+        dmax = warp_max_f32(dmax);
+        float best[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) best[c] = -CUDART_INF_F;
+        Vec<C> v[U];
+        float d[U];
+        // rows list[i .. i + U) into v, their deltas into d
+        auto load_rows = [&](int i) {
+#pragma unroll
+          for (int u = 0; u < U / 2; ++u) {
+            const float4 q = *reinterpret_cast<const float4*>(list + i + 2 * u);
+            const char* base = RES ? sA : gA;
+            const float* r0 = reinterpret_cast<const float*>(base + __float_as_int(q.y));
+            const float* r1 = reinterpret_cast<const float*>(base + __float_as_int(q.w));
+            if constexpr (RES) {
+              v[2 * u].lds(r0);
+              v[2 * u + 1].lds(r1);
+            } else {
+              v[2 * u].ldg(r0);
+              v[2 * u + 1].ldg(r1);
+            }
+            d[2 * u] = q.x;
+            d[2 * u + 1] = q.z;
+          }
+        };
+        auto use_rows = [&]() {
+#pragma unroll
+          for (int u = 0; u < U; u += 2)
+#pragma unroll
+            for (int c = 0; c < C; ++c)
+              best[c] = fmaxf(best[c], fmaxf(__fadd_rn(d[u], v[u].v[c]), __fadd_rn(d[u + 1], v[u + 1].v[c])));
+        };
+        // pads the list to whole groups with rows that give -inf
+        auto close_list = [&](int n) {
+          if (lane < U) list[n + lane] = make_float2(-CUDART_INF_F, 0.f);
+          __syncwarp();
+        };
+        // the listed rows (their order does not matter: only the maximum is kept)
+        auto flush = [&](int n) {
+          close_list(n);
+#pragma unroll 1
+          for (int i = 0; i < n; i += U) {
+            load_rows(i);
+            use_rows();
+          }
+          __syncwarp();
+        };
+        // the rows of the words kb .. kb + WB with lo <= delta < hi, after
+        // the n entries of the list; returns the new count
+        auto list_words = [&](int kb, float lo, float hi, int n) -> int {
+          if constexpr (!KEEP) {
+#pragma unroll
+            for (int k = 0; k < WB; ++k) dk[k] = dl[32 * (kb + k) + lane];
+          }
+#pragma unroll
+          for (int k = 0; k < WB; ++k) {
+            const bool in = dk[k] >= lo && dk[k] < hi;
+            const uint32_t mk = __ballot_sync(0xffffffffu, in);
+            if (in) list[n + __popc(mk & lt)] = make_float2(dk[k], __int_as_float((32 * (kb + k) + lane) * RB));
+            n += __popc(mk);
+          }
+          return n;
+        };
+        // pass 0: rows with delta >= dmax - gap.  The first group's loads are
+        // under way while the lists' candidates are formed.
+        float lo = fmaxf(__fmaf_rn(-0.85f, gap, dmax), -FLT_MAX);  // (never rows at -inf)
+        int n = 0;
+#pragma unroll 1
+        for (int kb = 0; kb < NW; kb += WB) {
+          n = list_words(kb, lo, CUDART_INF_F, n);
+          if (kb + WB < NW && n > CAP - 2 * U - 32 * WB) {
+            flush(n);
+            n = 0;
+          }
+        }
+        close_list(n);
+        load_rows(0);
+#pragma unroll
+        for (int x = 0; x < M; ++x)
+#pragma unroll
+          for (int c = 0; c < C; ++c) {
+            const uint32_t o = c % 2 ? lr[x][c / 2] >> 16 : lr[x][c / 2] & 0xffffu;
+            best[c] = fmaxf(best[c], __fadd_rn(*reinterpret_cast<const float*>(reinterpret_cast<const char*>(dl) + o),
+                                               lv[x][c]));
+          }
+        use_rows();
+#pragma unroll 1
+        for (int i = U; i < n; i += U) {
+          load_rows(i);
+          use_rows();
+        }
+        // pass 1: the rows below that which could still reach a target of
+        // this warp.  (A column without a finite weight outside its list
+        // gives NaN, which the minimum passes over.)
+        float th = CUDART_INF_F;
+#pragma unroll
+        for (int c = 0; c < C; ++c) th = fminf(th, need_delta(best[c], cut[c]));
+        th = warp_min_f32(th);
+        const float need = __fadd_rn(dmax, -th);
+        if (need < CUDART_INF_F && need >= 0.f) gap = 0.75f * gap + 0.25f * need;
+        if (th < lo) {
+          __syncwarp();
+          const float hi = lo;
+          lo = fmaxf(th, -FLT_MAX);
+          n = 0;
+#pragma unroll 1
+          for (int kb = 0; kb < NW; kb += WB) {
+            n = list_words(kb, lo, hi, n);
+            if (kb + WB >= NW || n > CAP - 2 * U - 32 * WB) {
+              flush(n);
+              n = 0;
+            }
+          }
+        }
+        bool zero = false;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          dval[c] = __fadd_rn(best[c], e[c]);  // (-inf beyond K)
+          zero = zero || dval[c] == 0.f;
+        }
+        if (zero) {
+          // a zero plus E = -0 has the sign of the kept candidate's zero,
+          // the lowest maximising row's
+#pragma unroll
+          for (int c = 0; c < C; ++c)
+            if (best[c] == 0.f && __float_as_uint(e[c]) == 0x80000000u && col0 + c < K)
+              for (int i = 0; i < K; ++i) {
+                const float x = __fadd_rn(dl[i], __ldg(a.pr_A + (int64_t)i * KP + col0 + c));
+                if (x == 0.f) {
+                  dval[c] = __fadd_rn(x, e[c]);
+                  break;
+                }
+              }
+        }
+      }
+      // ---- delta_t: shared memory (of every CTA of the cluster) and the table
+      float* dn = sd + cur * KP + col0;
+      if constexpr (C == 4) *reinterpret_cast<float4*>(dn) = make_float4(dval[0], dval[1], dval[2], dval[3]);
+      else if constexpr (C == 2) *reinterpret_cast<float2*>(dn) = make_float2(dval[0], dval[1]);
+      else dn[0] = dval[0];
+      if constexpr (CL > 1) {
+        const uint32_t bar = smem_addr(&s_bar[grp][cur]);
+        if (gt == 0) mbar_arrive_expect_tx(bar, (CL - 1) * KH * 4);
+        // 16 bytes per store: four lanes' columns where a lane has one
+        uint4 v = make_uint4(__float_as_uint(dval[0]), 0, 0, 0);
+        bool send = true;
+        int c4 = col0;
+        if constexpr (C == 4) {
+          v = make_uint4(__float_as_uint(dval[0]), __float_as_uint(dval[1]), __float_as_uint(dval[2]),
+                         __float_as_uint(dval[3]));
+        } else {
+          __syncwarp();
+          send = lane < 8 * C;
+          c4 = col0 - lane * C + 4 * (send ? lane : 0);
+          v = *reinterpret_cast<const uint4*>(sd + cur * KP + c4);
+        }
+        if (send) {
+          const uint32_t off = smem_addr(sd + cur * KP + c4) - self, boff = bar - self;
+#pragma unroll
+          for (int r = 0; r < CL; ++r)
+            if (r != (int)rank) st_async_v4(peer[r] + off, v, peer[r] + boff);
+        }
+      }
+      if (C > 1 && K % C == 0) {
+        if (col0 < K) {
+          if constexpr (C == 4) __stcs(reinterpret_cast<float4*>(dt), make_float4(dval[0], dval[1], dval[2], dval[3]));
+          if constexpr (C == 2) __stcs(reinterpret_cast<float2*>(dt), make_float2(dval[0], dval[1]));
+        }
+      } else {
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+          if (col0 + c < K) __stcs(dt + c, dval[c]);
+      }
+      dt += K;
+      bool late = false;
+      if constexpr (CL > 1) {
+        const uint32_t bar = smem_addr(&s_bar[grp][cur]), par = (ph >> 1) & 1u;
+        if (!mbar_try_wait_cluster(bar, par)) {
+          const long long w0 = clock64();
+          while (!late && !mbar_try_wait_cluster(bar, par))
+            late = *(volatile int*)&s_abort || clock64() - w0 > kPruneWaitCycles;
+        }
+      }
+      if (group_any(late)) {
+        // (cluster exchange only) a wait ran out: the job group stops; its
+        // own stores have landed by the end of the delay
+        set_status(a.hdr, FV_ETIMEOUT, 5);
+        *(volatile int*)&s_abort = 1;
+        const long long w0 = clock64();
+        while (clock64() - w0 < (1ll << 18)) {
+        }
+        live = false;
+        break;
+      }
+    }
+    if (!live) break;
+    if (rank == 0 && gw == 0) {
+      // termination: q_{T-1} = lowest argmax_j delta_{T-1}[j], score = delta_{T-1}[q]
+      const float* dl = sd + ((ph - 1u) & 1u) * KP;
+      float v = dl[lane];
+      int qi = lane;
+#pragma unroll
+      for (int k = 1; k < NW; ++k) {
+        const float vk = dl[lane + 32 * k];
+        if (vk > v) { v = vk; qi = lane + 32 * k; }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, v, o);
+        const int oq = __shfl_xor_sync(0xffffffffu, qi, o);
+        if (ov > v || (ov == v && oq < qi)) { v = ov; qi = oq; }
+      }
+      if (lane == 0) {
+        a.qlast[b] = qi;
+        a.scores[b] = dl[qi];
+      }
+    }
+  }
+  if constexpr (CL > 1) {
+    // no CTA leaves while another may still write to it or read its barriers
+    __syncwarp();
+    cluster_sync_all();
+  }
+}
+
+// ------------------------------------------------------------------ trace
+// The path from the stored deltas: q_{t-1} = lowest argmax_i of
+// fl(delta_{t-1}[i] + A[i][q_t]) -- only the path's own backpointers are
+// ever computed.  A step waits for a column of logA that depends on the
+// state before, so a sequence is cut into segments traced side by side: a
+// segment's trace starts kTraceWarm steps after its end from the best state
+// there (survivors of a Viterbi recursion meet within tens of steps), and a
+// second kernel follows the segments from the last one, which starts at the
+// known final state, and traces again from any end where the guess was not
+// the path's state until it meets the written path.
+constexpr int kTraceWarm = 24;
+
+template <int VPL>
+struct Tracer {
+  static constexpr int AH = VPL <= 8 ? 4 : 2;  // delta rows loaded ahead
+  const float* D;
+  const float* AT;
+  int K, KD, lane, slot;
+  float d[AH][VPL];
+  __device__ __forceinline__ void load(int t, float (&x)[VPL]) {
+#pragma unroll
+    for (int k = 0; k < VPL; ++k)
+      x[k] = (t >= 0 && 32 * k + lane < K) ? __ldcs(D + (int64_t)t * K + 32 * k + lane) : -CUDART_INF_F;
+  }
+  // rows t - 1, t - 2, ... for steps from state q_t downwards
+  __device__ __forceinline__ void start(int t) {
+#pragma unroll
+    for (int k = 0; k < AH; ++k) load(t - 1 - k, d[k]);
+  }
+  // lowest argmax over the lanes' (value, row); 0 where every value is -inf
+  __device__ __forceinline__ int lowest(float bv, int bi) {
+    const float m = warp_max_f32(__fadd_rn(bv, 0.f));  // (-0 as +0: they tie)
+    const uint32_t r = __reduce_min_sync(0xffffffffu, bv == m && bv > -CUDART_INF_F ? (uint32_t)bi : 0xffffffffu);
+    return r < (uint32_t)K ? (int)r : 0;
+  }
+  // q_{t-1} from q_t; `x` holds delta_{t-1} and receives row t - 1 - AH
+  __device__ __forceinline__ int step(int t, int q, float (&x)[VPL]) {
+    const float* col = AT + (int64_t)q * KD + lane;
+    float v[VPL];
+#pragma unroll
+    for (int k = 0; k < VPL; ++k) v[k] = 32 * k < KD ? __ldg(col + 32 * k) : -CUDART_INF_F;
+    float bv = -CUDART_INF_F;
+    int bi = 0;
+#pragma unroll
+    for (int k = 0; k < VPL; ++k) {
+      const float c = __fadd_rn(x[k], v[k]);
+      if (c > bv) { bv = c; bi = 32 * k + lane; }
+    }
+    load(t - 1 - AH, x);
+    return lowest(bv, bi);
+  }
+  // lowest argmax of delta_t
+  __device__ __forceinline__ int best(int t) {
+    float x[VPL];
+    load(t, x);
+    float bv = -CUDART_INF_F;
+    int bi = 0;
+#pragma unroll
+    for (int k = 0; k < VPL; ++k)
+      if (x[k] > bv) { bv = x[k]; bi = 32 * k + lane; }
+    return lowest(bv, bi);
+  }
+  // from q_t down to state `to`; f(time, state) returns true to stop there
+  template <typename F>
+  __device__ __forceinline__ int run(int t, int to, int q, F f) {
+    start(t);
+    while (t > to) {
+#pragma unroll
+      for (int s = 0; s < AH; ++s) {
+        if (t <= to) break;
+        q = step(t, q, d[s]);
+        --t;
+        if (f(t, q)) return q;
+      }
+    }
+    return q;
+  }
+};
+
+struct TraceArgs {
+  const Job* jobs;
+  const int32_t* order;
+  int32_t begin, count, K, seg;  // seg: states per segment
+  const float* D;
+  const float* AT;
+  const int32_t* qlast;
+  int32_t* paths;
+  int32_t* guess;  // state assumed at each segment's end
+  int64_t guess_cap;
+  const WsHeader* hdr;
+};
+// first guess of a sequence (at least ceil(T / seg) apart, as K > 128)
+__device__ __forceinline__ int64_t guess_off(const TraceArgs& a, const Job& jb, int b) {
+  return jb.aux_off / (128ll * a.seg) + b;
+}
+
+template <int VPL>
+__global__ void __launch_bounds__(32) prune_trace_kernel(TraceArgs a) {
+  if (a.hdr->status != 0) return;
+  const int b = a.order[a.begin + blockIdx.x];
+  const Job jb = a.jobs[b];
+  const int s = blockIdx.y, T = jb.T, K = a.K, lo = s * a.seg;
+  if (lo >= T) return;
+  Tracer<VPL> tr;
+  tr.D = a.D + jb.aux_off;
+  tr.AT = a.AT;
+  tr.K = K;
+  tr.KD = wide_lane_stride(K);
+  tr.lane = threadIdx.x;
+  int32_t* path = a.paths + jb.path_off;
+  const bool lead = threadIdx.x == 0;
+  int q = a.qlast[b];
+  q = (unsigned)q < (unsigned)K ? q : 0;
+  int t = T - 1;  // q = q_t
+  if (T - lo > a.seg) {
+    const int hi = lo + a.seg;  // hi <= T - 1
+    if (hi + kTraceWarm < T - 1) {
+      t = hi + kTraceWarm;
+      q = tr.best(t);
+    }
+    q = tr.run(t, hi, q, [](int, int) { return false; });
+    t = hi;
+    const int64_t g = guess_off(a, jb, b) + s;
+    if (lead && g < a.guess_cap) a.guess[g] = q;
+  } else if (lead) {
+    path[t] = q;
+  }
+  tr.run(t, lo, q, [&](int u, int x) {
+    if (lead) path[u] = x;
+    return false;
+  });
+}
+
+template <int VPL>
+__global__ void __launch_bounds__(32) prune_fix_kernel(TraceArgs a) {
+  if (a.hdr->status != 0) return;
+  const int b = a.order[a.begin + blockIdx.x], lane = threadIdx.x;
+  const Job jb = a.jobs[b];
+  const int K = a.K, nseg = (jb.T + a.seg - 1) / a.seg;
+  int32_t* path = a.paths + jb.path_off;
+  const int64_t g0 = guess_off(a, jb, b);
+  for (int s1 = nseg - 2; s1 >= 0;) {
+    // the highest of up to 32 segments s1, s1 - 1, ... whose end was guessed wrong
+    const int s = s1 - lane;
+    bool bad = false;
+    if (s >= 0) bad = g0 + s >= a.guess_cap || a.guess[g0 + s] != __ldcg(path + (int64_t)(s + 1) * a.seg);
+    const uint32_t m = __ballot_sync(0xffffffffu, bad);
+    if (!m) {
+      s1 -= 32;
+      continue;
+    }
+    const int sb = s1 - (__ffs(m) - 1), lo = sb * a.seg, hi = lo + a.seg;
+    Tracer<VPL> tr;
+    tr.D = a.D + jb.aux_off;
+    tr.AT = a.AT;
+    tr.K = K;
+    tr.KD = wide_lane_stride(K);
+    tr.lane = lane;
+    int q = __ldcg(path + hi);
+    q = (unsigned)q < (unsigned)K ? q : 0;
+    tr.run(hi, lo, q, [&](int u, int x) {
+      const bool same = __ldcg(path + u) == x;
+      __syncwarp();
+      if (!same && lane == 0) path[u] = x;
+      return same;
+    });
+    __syncwarp();
+    s1 = sb - 1;
+  }
+}
+
+// ---------------------------------------------------------------- launcher
+int prune_pad(int K) { return K <= 256 ? 256 : K <= 512 ? 512 : 1024; }
+// List lengths, from sweeps (us per step): K = 256, 4 / 6 entries: 1024
+// sequences 4.47 / 4.32 (two columns per lane); K = 512, 8 / 12: one sequence
+// 2.18 / 2.07; K = 1000, 8 / 12 / 16: 152 sequences 9.1 / 8.9 / 8.6.  A longer
+// list lowers the cutoffs (fewer rows) but gathers more deltas.
+int prune_list(int K) { return K <= 256 ? 6 : K <= 512 ? 12 : 16; }
+// area: row copy, column-major copy, list values, cutoffs, list rows
+size_t prune_area_bytes(int K) {
+  const size_t KP = prune_pad(K), M = prune_list(K);
+  return align_up((size_t)K * KP * 4) + align_up((size_t)K * wide_lane_stride(K) * 4) + align_up(KP * (M * 6 + 4));
+}
+
+template <int VPL>
+static cudaError_t launch_prep_cfg(const float* logA, int K, float* A, float* val, uint16_t* row, float* cut,
+                                   cudaStream_t st) {
+  const size_t sm = 8 * (32 * VPL + 4) * sizeof(float);
+  prune_prep_kernel<VPL><<<prune_pad(K) / 8, 256, sm, st>>>(logA, K, prune_pad(K), prune_list(K), A, val, row, cut);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_prune_prep(const float* logA, int K, char* area, DenseArgs* a, cudaStream_t st) {
+  const int KP = prune_pad(K), M = prune_list(K);
+  float* copy = reinterpret_cast<float*>(area);
+  area += align_up((size_t)K * KP * 4);
+  float* at = reinterpret_cast<float*>(area);
+  area += align_up((size_t)K * wide_lane_stride(K) * 4);
+  float* val = reinterpret_cast<float*>(area);
+  float* cut = val + (size_t)M * KP;
+  uint16_t* row = reinterpret_cast<uint16_t*>(cut + KP);
+  a->pr_A = copy;
+  a->pr_val = val;
+  a->pr_row = row;
+  a->pr_cut = cut;
+  a->wide_AT = at;
+  cudaError_t e = launch_wide_transpose(logA, K, at, st);
+  if (e != cudaSuccess) return e;
+  if (K <= 256) return launch_prep_cfg<8>(logA, K, copy, val, row, cut, st);
+  if (K <= 512) return launch_prep_cfg<16>(logA, K, copy, val, row, cut, st);
+  return launch_prep_cfg<32>(logA, K, copy, val, row, cut, st);
+}
+
+template <int KP, int CL, int C, int G, bool RES, int M>
+static cudaError_t launch_prune_cfg(const DenseArgs& a, cudaStream_t st) {
+  using Cfg = PruneCfg<KP, CL, C, G, RES, M>;
+  static_assert(Cfg::smem + 1024 <= 227 * 1024, "one CTA per SM");
+  static_assert(Cfg::W == 1 || G <= 15, "a named barrier per job group");
+  auto kern = prune_fwd_kernel<KP, CL, C, G, RES, M>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem);
+  if (e != cudaSuccess) return e;
+  const int nsm = device_sm_count(), jobs = a.order_count;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CL;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.blockDim = dim3(Cfg::NT);
+  cfg.dynamicSmemBytes = Cfg::smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int resident = 0;
+  if (CL > 1) {
+    cfg.gridDim = dim3(CL * nsm);
+    e = cudaOccupancyMaxActiveClusters(&resident, kern, &cfg);
+  } else {
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kern, Cfg::NT, Cfg::smem);
+    resident *= nsm;
+  }
+  if (e != cudaSuccess) return e;
+  if (resident < 1) return cudaErrorInvalidConfiguration;
+  cfg.gridDim = dim3(CL * (jobs < resident ? jobs : resident));
+  return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+// Configurations by state count and launch (GB300, us per step of the whole
+// call, Dirichlet(1) weights; the slot engine of fv_dense.cu in brackets):
+//   K <= 256, 2-CTA clusters, columns resident: two columns per lane and 8
+//     jobs per cluster 1.28 / 2.12 / 3.75 at 1 / 608 / 1024 equal sequences
+//     (2.29 / 6.78 / 11.6), four columns and 16 jobs 1.60 / 2.16 / 2.97.  Four
+//     columns spend less per job step but more per step of a lone job, so
+//     they are taken when the steps per SM outweigh the longest sequence
+//     (1024 sequences of 500 .. 4000 steps, which don't: 7.7 against 8.4 ms).
+//   K <= 512: one job per warp over 8-CTA clusters with resident columns
+//     while its slots (8 jobs on each of 15 clusters) hold the launch: 2.07 /
+//     2.46 at 1 / 64 sequences (3.47 / 4.27); then a CTA per job reading rows
+//     through L2: two columns per lane up to a job per SM, 3.6 at 152 (8.05),
+//     four columns and two CTAs per SM beyond, 4.8 at 304 (11.9).
+//   K <= 1024: a CTA per job: 6.2 / 6.8 at 1 / 152 (10.7 / 26.6).
+cudaError_t launch_prune_forward(const DenseArgs& a, int64_t sum_T, int max_T, cudaStream_t st) {
+  const int jobs = a.order_count, nsm = device_sm_count();
+  if (jobs <= 0) return cudaSuccess;
+  if (a.K <= 256) {
+    if (sum_T > 5ll * nsm * max_T) return launch_prune_cfg<256, 2, 4, 16, true, 6>(a, st);
+    return launch_prune_cfg<256, 2, 2, 8, true, 6>(a, st);
+  }
+  if (a.K <= 512) {
+    if (jobs <= 120) return launch_prune_cfg<512, 8, 2, 8, true, 12>(a, st);
+    if (jobs <= nsm) return launch_prune_cfg<512, 1, 2, 1, false, 12>(a, st);
+    return launch_prune_cfg<512, 1, 4, 1, false, 12>(a, st);
+  }
+  return launch_prune_cfg<1024, 1, 4, 1, false, 16>(a, st);
+}
+
+// States per segment of the trace: a few thousand segments over the launch,
+// each several times the warm-up.
+int prune_trace_seg(int64_t sum_T) {
+  const int64_t s = (sum_T / 4096 + 15) / 16 * 16;
+  return (int)(s < 48 ? 48 : s > 512 ? 512 : s);
+}
+size_t prune_guess_bytes(uint64_t aux_elems, int32_t n_seq, int64_t sum_T) {
+  return sizeof(int32_t) * (size_t)(aux_elems / (128ull * (uint64_t)prune_trace_seg(sum_T)) + (uint64_t)n_seq + 1ull);
+}
+
+template <int VPL>
+static cudaError_t launch_trace_cfg(const TraceArgs& t, int max_T, cudaStream_t st) {
+  const dim3 grid(t.count, (max_T + t.seg - 1) / t.seg);
+  prune_trace_kernel<VPL><<<grid, 32, 0, st>>>(t);
+  if (grid.y > 1) prune_fix_kernel<VPL><<<t.count, 32, 0, st>>>(t);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_prune_trace(const DenseArgs& a, int32_t* guess, size_t guess_bytes, int64_t sum_T, int max_T,
+                               int32_t* paths, cudaStream_t st) {
+  if (a.order_count <= 0) return cudaSuccess;
+  TraceArgs t;
+  t.jobs = a.jobs;
+  t.order = a.order;
+  t.begin = a.order_begin;
+  t.count = a.order_count;
+  t.K = a.K;
+  t.seg = prune_trace_seg(sum_T);
+  // (grid.y is at most 65535)
+  if (max_T / t.seg > 32768) t.seg = (max_T / 32768 + 1) * t.seg;
+  t.D = a.pr_D;
+  t.AT = a.wide_AT;
+  t.qlast = a.qlast;
+  t.paths = paths;
+  t.guess = guess;
+  t.guess_cap = (int64_t)(guess_bytes / sizeof(int32_t));
+  t.hdr = a.hdr;
+  if (a.K <= 256) return launch_trace_cfg<8>(t, max_T, st);
+  if (a.K <= 512) return launch_trace_cfg<16>(t, max_T, st);
+  return launch_trace_cfg<32>(t, max_T, st);
+}
+
+}  // namespace fv
