@@ -1447,7 +1447,7 @@ void dense_set_variant(int K, int v) {
 }
 int dense_get_variant(int K) { return g_variant[dense_k_class(K)]; }
 
-bool dense_prune_K(int K) { return K > 128 && K <= 1024; }
+bool dense_prune_K(int K) { return K > 128 && K <= 4096; }
 bool dense_uses_prune(int K, bool no_tune, bool withhold) {
   return dense_prune_K(K) && !withhold && (no_tune || g_variant[dense_k_class(K)] == 0);
 }

@@ -232,7 +232,7 @@ cudaError_t launch_wide_forward(DenseArgs a, cudaStream_t st);
 // small state spaces (K <= 128), every job kind: a CTA of K-class threads per
 // job, a thread per state (fv_small.cu)
 cudaError_t launch_small_forward(const DenseArgs& a, cudaStream_t st);
-// bounded-row engine (fv_prune.cu), exact decoding at 128 < K <= 1024: bytes
+// bounded-row engine (fv_prune.cu), exact decoding at 128 < K <= 4096: bytes
 // of a model's copies and column lists, their preparation, the forward
 // launch (delta rows to a.pr_D) and the backtrack from those rows
 size_t prune_area_bytes(int K);

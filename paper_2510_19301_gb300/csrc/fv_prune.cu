@@ -1,5 +1,5 @@
 // fv_prune.cu -- the exact forward engine with bounded candidate rows (exact
-// decoding, dense transitions, 128 < K <= 1024).
+// decoding, dense transitions, 128 < K <= 4096).
 //
 // The max-plus step (Sec. III-A) needs, for every target j, the maximum over
 // i of fl(delta[i] + A[i][j]).  Evaluating all K rows is bound by the FP32
@@ -23,8 +23,8 @@
 //
 // Measured (GB300): 1024 sequences of 500 .. 4000 steps, K = 256: 17.4 -> 7.7
 // ms per decode against the slot engine of fv_dense.cu; 150 sequences of 200
-// .. 1500 steps, K = 1000: 21.8 -> 8.7 ms; one K = 512 sequence of 512 steps:
-// 1.81 -> 1.34 ms.  Bound now: latency and shared-memory wavefronts (at K =
+// .. 1500 steps, K = 1000: 21.8 -> 7.3 ms; 8 sequences of 1500 steps, K = 4096:
+// 31.7 -> 17.3 ms; one K = 512 sequence of 512 steps: 1.81 -> 1.34 ms.  Bound now: latency and shared-memory wavefronts (at K =
 // 256, 650 wavefronts and 2200 warp instructions per job step), not the max.
 #include <cuda_runtime.h>
 #include <float.h>
@@ -170,6 +170,16 @@ struct Vec {
 };
 
 constexpr int kPruneAhead = 3;  // emission scores loaded this many steps ahead
+// The first row pass takes delta >= max(delta) - share x gap, gap a moving
+// mean of the depth that was needed: per warp (kGap), or for a common list
+// the largest depth of the job's warps here (kGapCommon; the second common
+// list reaches to kFarGap).  Measured: 0.75 / 0.85 / 1.0 / 1.15 of a warp's
+// own depth, 1024 K = 256 sequences, 7.91 / 7.78 / 7.88 / 8.42 ms; 0.85 / 0.95
+// / 1.05 of the largest, 150 K = 1000 sequences, 7.24 / 7.41 / 7.82 ms and 8 K
+// = 4096 sequences 17.6 / 17.1 / 18.4 ms; 0.85 / 1.0 of the mean depth 8.13 /
+// 7.62 and 18.6 / 17.4 ms.
+constexpr float kGap = 0.85f, kGapCommon = 0.9f, kFarGap = 1.3f;
+
 // KP = padded state count, CL = CTAs (a cluster) that split a job's columns,
 // C = adjacent columns per lane (a job takes W = KP / (32 CL C) warps of each
 // CTA), G = jobs side by side, RES = the CTA's columns of logA are resident
@@ -179,13 +189,18 @@ template <int KP, int CL, int C, int G, bool RES, int M>
 struct PruneCfg {
   static constexpr int KH = KP / CL, W = KH / (32 * C), NT = G * W * 32, NW = KP / 32;
   static constexpr int WB = NW < 8 ? NW : 8;  // words (of 32 rows) per list batch
-  static constexpr int U = RES ? 4 : 8;       // rows in flight (shared memory / L2 latency)
+  static constexpr int U = RES ? 4 : (C <= 2 ? 16 : 8);  // rows in flight (shared memory / L2 latency)
   // row list entries of a warp (a batch may add 32 WB to a list that is not yet full)
   static constexpr int CAP = (NW <= WB ? KP : 32 * WB + 128) + 2 * U;
   static constexpr size_t a_bytes = RES ? (size_t)KP * KH * 4 : 0;
   static constexpr size_t d_bytes = (size_t)G * 2 * KP * 4;  // delta, double buffered
   static constexpr size_t l_bytes = (size_t)G * W * CAP * 8;
-  static constexpr size_t smem = a_bytes + d_bytes + l_bytes;
+  // COOP: the warps of a job build the first row list together, and a second
+  // one of the rows the later pass is likely to want
+  static constexpr bool COOP = W > 1 && NW > 8;
+  static constexpr int NL = KP + U;  // entries of a common list
+  static constexpr size_t s_bytes = COOP ? (size_t)G * 2 * NL * 8 : 0;
+  static constexpr size_t smem = a_bytes + d_bytes + l_bytes + s_bytes;
 };
 // bounded wait of the cluster exchange (~1 s at 2 GHz)
 constexpr long long kPruneWaitCycles = 1ll << 31;
@@ -194,10 +209,13 @@ template <int KP, int CL, int C, int G, bool RES, int M>
 __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_fwd_kernel(DenseArgs a) {
   using Cfg = PruneCfg<KP, CL, C, G, RES, M>;
   constexpr int KH = Cfg::KH, W = Cfg::W, NT = Cfg::NT, NW = Cfg::NW, CAP = Cfg::CAP, WB = Cfg::WB, U = Cfg::U;
+  constexpr bool COOP = Cfg::COOP;
   extern __shared__ __align__(16) char smem[];
   __shared__ __align__(8) uint64_t s_bar[G][2];
   __shared__ int s_abort;
   __shared__ uint32_t s_stop[CL];
+  __shared__ float s_max[G][W], s_need[G][2][W];  // COOP: per warp maxima and depths
+  __shared__ int s_cnt[G][2][2];                  // COOP: entries of the common lists, by step parity
   const bool stop = a.hdr->status != 0;  // an earlier kernel recorded an error
   if (CL == 1 && stop) return;
   const int K = a.K;
@@ -209,6 +227,8 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
   char* sA = smem + gt * C * 4;
   float* sd = reinterpret_cast<float*>(smem + Cfg::a_bytes) + grp * 2 * KP;
   float2* list = reinterpret_cast<float2*>(smem + Cfg::a_bytes + Cfg::d_bytes) + warp * CAP;
+  float2* near = reinterpret_cast<float2*>(smem + Cfg::a_bytes + Cfg::d_bytes + Cfg::l_bytes) + grp * 2 * Cfg::NL;
+  float2* far = near + Cfg::NL;
   // barrier of the job's warps here; true where any thread passes true
   auto group_any = [&](bool x) -> bool {
     if constexpr (W == 1) {
@@ -245,12 +265,14 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
     }
 #pragma unroll
   for (int c = 0; c < C; ++c) cut[c] = __ldg(a.pr_cut + col0 + c);
-  uint32_t peer[CL];  // the other CTAs' shared memory
+  uint32_t peer[2] = {0u, 0u};  // CL = 2: shared memory of either CTA
   const uint32_t self = smem_addr(smem);
   if (threadIdx.x == 0) s_abort = 0;
   if constexpr (CL > 1) {
-#pragma unroll
-    for (int r = 0; r < CL; ++r) peer[r] = dsmem_addr(smem, r);
+    if constexpr (CL == 2) {
+      peer[0] = dsmem_addr(smem, 0);
+      peer[1] = dsmem_addr(smem, 1);
+    }
     if (threadIdx.x < 2 * G) {
       mbar_init(smem_addr(&s_bar[0][0] + threadIdx.x), 1);
       fence_mbar_init_cluster();
@@ -331,29 +353,78 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
       float dval[C];
       const float* dl = sd + (cur ^ 1u) * KP;
       if (t == 0) {
+        if (COOP && lane == 0) s_need[grp][cur][gw] = -1.f;
 #pragma unroll
         for (int c = 0; c < C; ++c)
           dval[c] = col0 + c < K ? __fadd_rn(__ldg(a.log_pi + col0 + c), e[c]) : -CUDART_INF_F;
       } else {
-        constexpr bool KEEP = NW <= 8;  // the deltas of this lane stay in registers
-        float dk[WB], dmax = -CUDART_INF_F;
+        constexpr bool KEEP = NW <= 8;          // the deltas of this lane stay in registers
+        constexpr int NK = COOP ? NW / W : NW;  // words this warp looks over for the maximum
+        float dk[COOP && NK > WB ? NK : WB], dmax = -CUDART_INF_F;
 #pragma unroll
-        for (int k = 0; k < NW; ++k) {
-          const float d = dl[32 * k + lane];
-          if constexpr (KEEP) dk[k] = d;
+        for (int k = 0; k < NK; ++k) {
+          const float d = dl[32 * (COOP ? gw * NK + k : k) + lane];
+          if constexpr (KEEP || COOP) dk[k] = d;
           dmax = fmaxf(dmax, d);
         }
         dmax = warp_max_f32(dmax);
+        float lo, lo1 = 0.f;  // pass 0 takes delta >= lo; the second common list lo1 <= delta < lo
+        int n = 0, n1 = 0;
+        if constexpr (COOP) {
+          if (lane == 0) s_max[grp][gw] = dmax;
+          if (gt < 2) s_cnt[grp][cur][gt] = 0;
+          group_any(false);
+          float most = -1.f;
+#pragma unroll
+          for (int w = 0; w < W; ++w) {
+            dmax = fmaxf(dmax, s_max[grp][w]);
+            const float x = s_need[grp][cur ^ 1u][w];
+            most = fmaxf(most, x);
+          }
+          if (most >= 0.f) gap = 0.75f * gap + 0.25f * most;
+          lo = fmaxf(__fmaf_rn(-kGapCommon, gap, dmax), -FLT_MAX);  // (never rows at -inf)
+          lo1 = fmaxf(__fmaf_rn(-kFarGap, gap, dmax), -FLT_MAX);
+          // this lane's rows of either list (low and high half), their
+          // places by a scan over the lanes and one add per warp and list
+          uint32_t c = 0;
+#pragma unroll
+          for (int k = 0; k < NK; ++k) c += dk[k] >= lo ? 1u : (dk[k] >= lo1 ? 0x10000u : 0u);
+          uint32_t x = c;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+          }
+          uint32_t base = 0;
+          const uint32_t tot = __shfl_sync(0xffffffffu, x, 31);
+          if (lane >= 30) base = (uint32_t)atomicAdd(&s_cnt[grp][cur][lane - 30], (int)(lane == 30 ? tot & 0xffffu : tot >> 16));
+          int p0 = (int)(__shfl_sync(0xffffffffu, base, 30) + ((x - c) & 0xffffu));
+          int p1 = (int)(__shfl_sync(0xffffffffu, base, 31) + ((x - c) >> 16));
+#pragma unroll
+          for (int k = 0; k < NK; ++k) {
+            const float2 ent = make_float2(dk[k], __int_as_float((32 * (gw * NK + k) + lane) * RB));
+            const bool i0 = dk[k] >= lo, i1 = !i0 && dk[k] >= lo1;
+            float2* to = i0 ? near + p0 : far + p1;
+            if (i0 || i1) *to = ent;
+            p0 += i0;
+            p1 += i1;
+          }
+          group_any(false);
+          n = s_cnt[grp][cur][0];
+          n1 = s_cnt[grp][cur][1];
+        } else {
+          lo = fmaxf(__fmaf_rn(-kGap, gap, dmax), -FLT_MAX);  // (never rows at -inf)
+        }
         float best[C];
 #pragma unroll
         for (int c = 0; c < C; ++c) best[c] = -CUDART_INF_F;
         Vec<C> v[U];
         float d[U];
-        // rows list[i .. i + U) into v, their deltas into d
-        auto load_rows = [&](int i) {
+        // rows src[i .. i + U) into v, their deltas into d
+        auto load_rows = [&](const float2* src, int i) {
 #pragma unroll
           for (int u = 0; u < U / 2; ++u) {
-            const float4 q = *reinterpret_cast<const float4*>(list + i + 2 * u);
+            const float4 q = *reinterpret_cast<const float4*>(src + i + 2 * u);
             const char* base = RES ? sA : gA;
             const float* r0 = reinterpret_cast<const float*>(base + __float_as_int(q.y));
             const float* r1 = reinterpret_cast<const float*>(base + __float_as_int(q.w));
@@ -376,16 +447,16 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
               best[c] = fmaxf(best[c], fmaxf(__fadd_rn(d[u], v[u].v[c]), __fadd_rn(d[u + 1], v[u + 1].v[c])));
         };
         // pads the list to whole groups with rows that give -inf
-        auto close_list = [&](int n) {
-          if (lane < U) list[n + lane] = make_float2(-CUDART_INF_F, 0.f);
+        auto close_list = [&](float2* src, int n) {
+          if (lane < U) src[n + lane] = make_float2(-CUDART_INF_F, 0.f);
           __syncwarp();
         };
         // the listed rows (their order does not matter: only the maximum is kept)
         auto flush = [&](int n) {
-          close_list(n);
+          close_list(list, n);
 #pragma unroll 1
           for (int i = 0; i < n; i += U) {
-            load_rows(i);
+            load_rows(list, i);
             use_rows();
           }
           __syncwarp();
@@ -408,18 +479,19 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
         };
         // pass 0: rows with delta >= dmax - gap.  The first group's loads are
         // under way while the lists' candidates are formed.
-        float lo = fmaxf(__fmaf_rn(-0.85f, gap, dmax), -FLT_MAX);  // (never rows at -inf)
-        int n = 0;
+        float2* const first = COOP ? near : list;
+        if constexpr (!COOP) {
 #pragma unroll 1
-        for (int kb = 0; kb < NW; kb += WB) {
-          n = list_words(kb, lo, CUDART_INF_F, n);
-          if (kb + WB < NW && n > CAP - 2 * U - 32 * WB) {
-            flush(n);
-            n = 0;
+          for (int kb = 0; kb < NW; kb += WB) {
+            n = list_words(kb, lo, CUDART_INF_F, n);
+            if (kb + WB < NW && n > CAP - 2 * U - 32 * WB) {
+              flush(n);
+              n = 0;
+            }
           }
         }
-        close_list(n);
-        load_rows(0);
+        close_list(first, n);  // (every warp writes the same beyond a common list)
+        load_rows(first, 0);
 #pragma unroll
         for (int x = 0; x < M; ++x)
 #pragma unroll
@@ -431,7 +503,7 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
         use_rows();
 #pragma unroll 1
         for (int i = U; i < n; i += U) {
-          load_rows(i);
+          load_rows(first, i);
           use_rows();
         }
         // pass 1: the rows below that which could still reach a target of
@@ -442,18 +514,41 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
         for (int c = 0; c < C; ++c) th = fminf(th, need_delta(best[c], cut[c]));
         th = warp_min_f32(th);
         const float need = __fadd_rn(dmax, -th);
-        if (need < CUDART_INF_F && need >= 0.f) gap = 0.75f * gap + 0.25f * need;
+        const bool depth = need < CUDART_INF_F && need >= 0.f;
+        if constexpr (COOP) {
+          if (lane == 0) s_need[grp][cur][gw] = depth ? need : -1.f;
+        } else {
+          if (depth) gap = 0.75f * gap + 0.25f * need;
+        }
         if (th < lo) {
           __syncwarp();
-          const float hi = lo;
-          lo = fmaxf(th, -FLT_MAX);
-          n = 0;
+          if (COOP && th >= lo1) {
+            // the second common list holds them
+            n = 0;
 #pragma unroll 1
-          for (int kb = 0; kb < NW; kb += WB) {
-            n = list_words(kb, lo, hi, n);
-            if (kb + WB >= NW || n > CAP - 2 * U - 32 * WB) {
-              flush(n);
-              n = 0;
+            for (int i0 = 0; i0 < n1; i0 += 32) {
+              const bool have = i0 + lane < n1;
+              const float2 ent = far[have ? i0 + lane : 0];
+              const bool in = have && ent.x >= th;
+              const uint32_t mk = __ballot_sync(0xffffffffu, in);
+              if (in) list[n + __popc(mk & lt)] = ent;
+              n += __popc(mk);
+              if (i0 + 32 >= n1 || n > CAP - 2 * U - 32) {
+                flush(n);
+                n = 0;
+              }
+            }
+          } else {
+            const float hi = lo;
+            lo = fmaxf(th, -FLT_MAX);
+            n = 0;
+#pragma unroll 1
+            for (int kb = 0; kb < NW; kb += WB) {
+              n = list_words(kb, lo, hi, n);
+              if (kb + WB >= NW || n > CAP - 2 * U - 32 * WB) {
+                flush(n);
+                n = 0;
+              }
             }
           }
         }
@@ -486,24 +581,38 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
       if constexpr (CL > 1) {
         const uint32_t bar = smem_addr(&s_bar[grp][cur]);
         if (gt == 0) mbar_arrive_expect_tx(bar, (CL - 1) * KH * 4);
-        // 16 bytes per store: four lanes' columns where a lane has one
-        uint4 v = make_uint4(__float_as_uint(dval[0]), 0, 0, 0);
-        bool send = true;
-        int c4 = col0;
-        if constexpr (C == 4) {
-          v = make_uint4(__float_as_uint(dval[0]), __float_as_uint(dval[1]), __float_as_uint(dval[2]),
-                         __float_as_uint(dval[3]));
+        if constexpr (CL == 2) {
+          // 16 bytes per store: four lanes' columns where a lane has one
+          uint4 v = make_uint4(__float_as_uint(dval[0]), 0, 0, 0);
+          bool send = true;
+          int c4 = col0;
+          if constexpr (C == 4) {
+            v = make_uint4(__float_as_uint(dval[0]), __float_as_uint(dval[1]), __float_as_uint(dval[2]),
+                           __float_as_uint(dval[3]));
+          } else {
+            __syncwarp();
+            send = lane < 8 * C;
+            c4 = col0 - lane * C + 4 * (send ? lane : 0);
+            v = *reinterpret_cast<const uint4*>(sd + cur * KP + c4);
+          }
+          if (send) {
+            const uint32_t off = smem_addr(sd + cur * KP + c4) - self, boff = bar - self;
+            const uint32_t to = rank ? peer[0] : peer[1];
+            st_async_v4(to + off, v, to + boff);
+          }
         } else {
-          __syncwarp();
-          send = lane < 8 * C;
-          c4 = col0 - lane * C + 4 * (send ? lane : 0);
-          v = *reinterpret_cast<const uint4*>(sd + cur * KP + c4);
-        }
-        if (send) {
-          const uint32_t off = smem_addr(sd + cur * KP + c4) - self, boff = bar - self;
-#pragma unroll
-          for (int r = 0; r < CL; ++r)
-            if (r != (int)rank) st_async_v4(peer[r] + off, v, peer[r] + boff);
+          // one copy of the CTA's columns to each of the others
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          group_any(false);
+          if (gt < CL && gt != (int)rank) {
+            const uint32_t src = smem_addr(sd + cur * KP + (int)rank * KH);
+            const uint32_t to = dsmem_addr(smem, gt);
+            asm volatile(
+                "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                    to + (src - self)),
+                "r"(src), "r"(KH * 4), "r"(to + (bar - self))
+                : "memory");
+          }
         }
       }
       if (C > 1 && K % C == 0) {
@@ -580,41 +689,69 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
 // the path's state until it meets the written path.
 constexpr int kTraceWarm = 24;
 
-template <int VPL>
+// TW warps of a CTA follow one chain, VPL rows of a column per thread.
+template <int VPL, int TW>
 struct Tracer {
   static constexpr int AH = VPL <= 8 ? 4 : 2;  // delta rows loaded ahead
+  static constexpr int NT = 32 * TW;
   const float* D;
   const float* AT;
-  int K, KD, lane, slot;
+  int K, KD, tid;
+  uint2* part;  // shared, [2][TW]: per warp (value, row) of a step, by turns
+  int turn;
   float d[AH][VPL];
+  __device__ __forceinline__ void init(const float* D_, const float* AT_, int K_, uint2* part_) {
+    D = D_;
+    AT = AT_;
+    K = K_;
+    KD = wide_lane_stride(K_);
+    tid = threadIdx.x;
+    part = part_;
+    turn = 0;
+  }
   __device__ __forceinline__ void load(int t, float (&x)[VPL]) {
 #pragma unroll
     for (int k = 0; k < VPL; ++k)
-      x[k] = (t >= 0 && 32 * k + lane < K) ? __ldcs(D + (int64_t)t * K + 32 * k + lane) : -CUDART_INF_F;
+      x[k] = (t >= 0 && NT * k + tid < K) ? __ldcs(D + (int64_t)t * K + NT * k + tid) : -CUDART_INF_F;
   }
   // rows t - 1, t - 2, ... for steps from state q_t downwards
   __device__ __forceinline__ void start(int t) {
 #pragma unroll
     for (int k = 0; k < AH; ++k) load(t - 1 - k, d[k]);
   }
-  // lowest argmax over the lanes' (value, row); 0 where every value is -inf
+  // lowest argmax over the threads' (value, row); 0 where every value is -inf
   __device__ __forceinline__ int lowest(float bv, int bi) {
-    const float m = warp_max_f32(__fadd_rn(bv, 0.f));  // (-0 as +0: they tie)
-    const uint32_t r = __reduce_min_sync(0xffffffffu, bv == m && bv > -CUDART_INF_F ? (uint32_t)bi : 0xffffffffu);
+    float v = __fadd_rn(bv, 0.f);  // (-0 as +0: they tie)
+    float m = warp_max_f32(v);
+    uint32_t r = __reduce_min_sync(0xffffffffu, v == m && v > -CUDART_INF_F ? (uint32_t)bi : 0xffffffffu);
+    if constexpr (TW > 1) {
+      if ((tid & 31) == 0) part[turn * TW + tid / 32] = make_uint2(__float_as_uint(m), r);
+      __syncthreads();
+#pragma unroll
+      for (int w = 0; w < TW; ++w) {
+        const uint2 x = part[turn * TW + w];
+        const float y = __uint_as_float(x.x);
+        if (w == 0 || y > m || (y == m && x.y < r)) {
+          m = y;
+          r = x.y;
+        }
+      }
+      turn ^= 1;
+    }
     return r < (uint32_t)K ? (int)r : 0;
   }
   // q_{t-1} from q_t; `x` holds delta_{t-1} and receives row t - 1 - AH
   __device__ __forceinline__ int step(int t, int q, float (&x)[VPL]) {
-    const float* col = AT + (int64_t)q * KD + lane;
+    const float* col = AT + (int64_t)q * KD + tid;
     float v[VPL];
 #pragma unroll
-    for (int k = 0; k < VPL; ++k) v[k] = 32 * k < KD ? __ldg(col + 32 * k) : -CUDART_INF_F;
+    for (int k = 0; k < VPL; ++k) v[k] = NT * k + tid < KD ? __ldg(col + NT * k) : -CUDART_INF_F;
     float bv = -CUDART_INF_F;
     int bi = 0;
 #pragma unroll
     for (int k = 0; k < VPL; ++k) {
       const float c = __fadd_rn(x[k], v[k]);
-      if (c > bv) { bv = c; bi = 32 * k + lane; }
+      if (c > bv) { bv = c; bi = NT * k + tid; }
     }
     load(t - 1 - AH, x);
     return lowest(bv, bi);
@@ -627,7 +764,7 @@ struct Tracer {
     int bi = 0;
 #pragma unroll
     for (int k = 0; k < VPL; ++k)
-      if (x[k] > bv) { bv = x[k]; bi = 32 * k + lane; }
+      if (x[k] > bv) { bv = x[k]; bi = NT * k + tid; }
     return lowest(bv, bi);
   }
   // from q_t down to state `to`; f(time, state) returns true to stop there
@@ -664,19 +801,16 @@ __device__ __forceinline__ int64_t guess_off(const TraceArgs& a, const Job& jb, 
   return jb.aux_off / (128ll * a.seg) + b;
 }
 
-template <int VPL>
-__global__ void __launch_bounds__(32) prune_trace_kernel(TraceArgs a) {
+template <int VPL, int TW>
+__global__ void __launch_bounds__(32 * TW) prune_trace_kernel(TraceArgs a) {
+  __shared__ uint2 part[2 * TW];
   if (a.hdr->status != 0) return;
   const int b = a.order[a.begin + blockIdx.x];
   const Job jb = a.jobs[b];
   const int s = blockIdx.y, T = jb.T, K = a.K, lo = s * a.seg;
   if (lo >= T) return;
-  Tracer<VPL> tr;
-  tr.D = a.D + jb.aux_off;
-  tr.AT = a.AT;
-  tr.K = K;
-  tr.KD = wide_lane_stride(K);
-  tr.lane = threadIdx.x;
+  Tracer<VPL, TW> tr;
+  tr.init(a.D + jb.aux_off, a.AT, K, part);
   int32_t* path = a.paths + jb.path_off;
   const bool lead = threadIdx.x == 0;
   int q = a.qlast[b];
@@ -701,16 +835,22 @@ __global__ void __launch_bounds__(32) prune_trace_kernel(TraceArgs a) {
   });
 }
 
-template <int VPL>
-__global__ void __launch_bounds__(32) prune_fix_kernel(TraceArgs a) {
+template <int VPL, int TW>
+__global__ void __launch_bounds__(32 * TW) prune_fix_kernel(TraceArgs a) {
+  __shared__ uint2 part[2 * TW];
   if (a.hdr->status != 0) return;
-  const int b = a.order[a.begin + blockIdx.x], lane = threadIdx.x;
+  const int b = a.order[a.begin + blockIdx.x], lane = threadIdx.x & 31;
   const Job jb = a.jobs[b];
   const int K = a.K, nseg = (jb.T + a.seg - 1) / a.seg;
   int32_t* path = a.paths + jb.path_off;
   const int64_t g0 = guess_off(a, jb, b);
+  auto sync = []() {
+    if constexpr (TW > 1) __syncthreads();
+    else __syncwarp();
+  };
   for (int s1 = nseg - 2; s1 >= 0;) {
-    // the highest of up to 32 segments s1, s1 - 1, ... whose end was guessed wrong
+    // the highest of up to 32 segments s1, s1 - 1, ... whose end was guessed
+    // wrong (every warp finds the same)
     const int s = s1 - lane;
     bool bad = false;
     if (s >= 0) bad = g0 + s >= a.guess_cap || a.guess[g0 + s] != __ldcg(path + (int64_t)(s + 1) * a.seg);
@@ -720,32 +860,29 @@ __global__ void __launch_bounds__(32) prune_fix_kernel(TraceArgs a) {
       continue;
     }
     const int sb = s1 - (__ffs(m) - 1), lo = sb * a.seg, hi = lo + a.seg;
-    Tracer<VPL> tr;
-    tr.D = a.D + jb.aux_off;
-    tr.AT = a.AT;
-    tr.K = K;
-    tr.KD = wide_lane_stride(K);
-    tr.lane = lane;
+    Tracer<VPL, TW> tr;
+    tr.init(a.D + jb.aux_off, a.AT, K, part);
     int q = __ldcg(path + hi);
     q = (unsigned)q < (unsigned)K ? q : 0;
+    sync();
     tr.run(hi, lo, q, [&](int u, int x) {
       const bool same = __ldcg(path + u) == x;
-      __syncwarp();
-      if (!same && lane == 0) path[u] = x;
+      sync();
+      if (!same && threadIdx.x == 0) path[u] = x;
       return same;
     });
-    __syncwarp();
+    __threadfence_block();
+    sync();
     s1 = sb - 1;
   }
 }
 
-// ---------------------------------------------------------------- launcher
-int prune_pad(int K) { return K <= 256 ? 256 : K <= 512 ? 512 : 1024; }
+int prune_pad(int K) { return K <= 256 ? 256 : K <= 512 ? 512 : K <= 1024 ? 1024 : K <= 2048 ? 2048 : 4096; }
 // List lengths, from sweeps (us per step): K = 256, 4 / 6 entries: 1024
 // sequences 4.47 / 4.32 (two columns per lane); K = 512, 8 / 12: one sequence
 // 2.18 / 2.07; K = 1000, 8 / 12 / 16: 152 sequences 9.1 / 8.9 / 8.6.  A longer
 // list lowers the cutoffs (fewer rows) but gathers more deltas.
-int prune_list(int K) { return K <= 256 ? 6 : K <= 512 ? 12 : 16; }
+int prune_list(int K) { return K <= 256 ? 6 : K <= 512 ? 12 : K <= 1024 ? 16 : 32; }
 // area: row copy, column-major copy, list values, cutoffs, list rows
 size_t prune_area_bytes(int K) {
   const size_t KP = prune_pad(K), M = prune_list(K);
@@ -756,6 +893,9 @@ template <int VPL>
 static cudaError_t launch_prep_cfg(const float* logA, int K, float* A, float* val, uint16_t* row, float* cut,
                                    cudaStream_t st) {
   const size_t sm = 8 * (32 * VPL + 4) * sizeof(float);
+  cudaError_t e =
+      cudaFuncSetAttribute(prune_prep_kernel<VPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
   prune_prep_kernel<VPL><<<prune_pad(K) / 8, 256, sm, st>>>(logA, K, prune_pad(K), prune_list(K), A, val, row, cut);
   return cudaGetLastError();
 }
@@ -778,41 +918,56 @@ cudaError_t launch_prune_prep(const float* logA, int K, char* area, DenseArgs* a
   if (e != cudaSuccess) return e;
   if (K <= 256) return launch_prep_cfg<8>(logA, K, copy, val, row, cut, st);
   if (K <= 512) return launch_prep_cfg<16>(logA, K, copy, val, row, cut, st);
-  return launch_prep_cfg<32>(logA, K, copy, val, row, cut, st);
+  if (K <= 1024) return launch_prep_cfg<32>(logA, K, copy, val, row, cut, st);
+  if (K <= 2048) return launch_prep_cfg<64>(logA, K, copy, val, row, cut, st);
+  return launch_prep_cfg<128>(logA, K, copy, val, row, cut, st);
 }
 
+// Clusters (CTAs for CL = 1) of a configuration resident at once; 0 where the
+// device does not take it.
 template <int KP, int CL, int C, int G, bool RES, int M>
-static cudaError_t launch_prune_cfg(const DenseArgs& a, cudaStream_t st) {
+static int prune_resident(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
   using Cfg = PruneCfg<KP, CL, C, G, RES, M>;
   static_assert(Cfg::smem + 1024 <= 227 * 1024, "one CTA per SM");
   static_assert(Cfg::W == 1 || G <= 15, "a named barrier per job group");
   auto kern = prune_fwd_kernel<KP, CL, C, G, RES, M>;
+  int n = 0;
+  const int nsm = device_sm_count();
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = CL;
+  attr->val.clusterDim.y = 1;
+  attr->val.clusterDim.z = 1;
+  cfg->gridDim = dim3(CL * nsm);
+  cfg->blockDim = dim3(Cfg::NT);
+  cfg->dynamicSmemBytes = Cfg::smem;
+  cfg->attrs = attr;
+  cfg->numAttrs = 1;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem);
-  if (e != cudaSuccess) return e;
-  const int nsm = device_sm_count(), jobs = a.order_count;
+  if (e == cudaSuccess && CL > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess) {
+    if (CL > 1) {
+      e = cudaOccupancyMaxActiveClusters(&n, kern, cfg);
+    } else {
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, Cfg::NT, Cfg::smem);
+      n *= nsm;
+    }
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+template <int KP, int CL, int C, int G, bool RES, int M>
+static cudaError_t launch_prune_cfg(const DenseArgs& a, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CL;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.blockDim = dim3(Cfg::NT);
-  cfg.dynamicSmemBytes = Cfg::smem;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int resident = 0;
-  if (CL > 1) {
-    cfg.gridDim = dim3(CL * nsm);
-    e = cudaOccupancyMaxActiveClusters(&resident, kern, &cfg);
-  } else {
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kern, Cfg::NT, Cfg::smem);
-    resident *= nsm;
-  }
-  if (e != cudaSuccess) return e;
+  const int resident = prune_resident<KP, CL, C, G, RES, M>(&cfg, attr), jobs = a.order_count;
   if (resident < 1) return cudaErrorInvalidConfiguration;
+  cfg.stream = st;
   cfg.gridDim = dim3(CL * (jobs < resident ? jobs : resident));
-  return cudaLaunchKernelEx(&cfg, kern, a);
+  return cudaLaunchKernelEx(&cfg, prune_fwd_kernel<KP, CL, C, G, RES, M>, a);
 }
 
 // Configurations by state count and launch (GB300, us per step of the whole
@@ -828,7 +983,15 @@ static cudaError_t launch_prune_cfg(const DenseArgs& a, cudaStream_t st) {
 //     2.46 at 1 / 64 sequences (3.47 / 4.27); then a CTA per job reading rows
 //     through L2: two columns per lane up to a job per SM, 3.6 at 152 (8.05),
 //     four columns and two CTAs per SM beyond, 4.8 at 304 (11.9).
-//   K <= 1024: a CTA per job: 6.2 / 6.8 at 1 / 152 (10.7 / 26.6).
+//   K <= 1024: a CTA per job, 5.9 at 152 (26.6), bound by the L2 reads of its
+//     rows (64 bytes per clock); half as many jobs take two CTAs each, 3.7 at
+//     40 (10.7; four CTAs 4.1, eight 3.8).
+//   K <= 2048: 4-CTA clusters, 5.1 at 1 .. 30 sequences (eight CTAs 5.3 up to
+//     15 sequences); K <= 4096: 8-CTA clusters, 15 at a time, 8.7 at 8 (21.1 on
+//     the whole-GPU engine of fv_wide.cu, which reads all of logA every step;
+//     16-CTA clusters fit seven at a time and took 21.8).  512 columns per CTA,
+//     two per lane (one per lane: 6.7 and 11.8).  List lengths 24 / 32 / 48 at
+//     K = 4096, 8 sequences with Dirichlet(0.1) rows: 21.6 / 17.3 / 28.0 ms.
 cudaError_t launch_prune_forward(const DenseArgs& a, int64_t sum_T, int max_T, cudaStream_t st) {
   const int jobs = a.order_count, nsm = device_sm_count();
   if (jobs <= 0) return cudaSuccess;
@@ -841,7 +1004,12 @@ cudaError_t launch_prune_forward(const DenseArgs& a, int64_t sum_T, int max_T, c
     if (jobs <= nsm) return launch_prune_cfg<512, 1, 2, 1, false, 12>(a, st);
     return launch_prune_cfg<512, 1, 4, 1, false, 12>(a, st);
   }
-  return launch_prune_cfg<1024, 1, 4, 1, false, 16>(a, st);
+  if (a.K <= 1024) {
+    if (2 * jobs <= nsm) return launch_prune_cfg<1024, 2, 2, 1, false, 16>(a, st);
+    return launch_prune_cfg<1024, 1, 4, 1, false, 16>(a, st);
+  }
+  if (a.K <= 2048) return launch_prune_cfg<2048, 4, 2, 1, false, 32>(a, st);
+  return launch_prune_cfg<4096, 8, 2, 1, false, 32>(a, st);
 }
 
 // States per segment of the trace: a few thousand segments over the launch,
@@ -854,11 +1022,11 @@ size_t prune_guess_bytes(uint64_t aux_elems, int32_t n_seq, int64_t sum_T) {
   return sizeof(int32_t) * (size_t)(aux_elems / (128ull * (uint64_t)prune_trace_seg(sum_T)) + (uint64_t)n_seq + 1ull);
 }
 
-template <int VPL>
+template <int VPL, int TW>
 static cudaError_t launch_trace_cfg(const TraceArgs& t, int max_T, cudaStream_t st) {
   const dim3 grid(t.count, (max_T + t.seg - 1) / t.seg);
-  prune_trace_kernel<VPL><<<grid, 32, 0, st>>>(t);
-  if (grid.y > 1) prune_fix_kernel<VPL><<<t.count, 32, 0, st>>>(t);
+  prune_trace_kernel<VPL, TW><<<grid, 32 * TW, 0, st>>>(t);
+  if (grid.y > 1) prune_fix_kernel<VPL, TW><<<t.count, 32 * TW, 0, st>>>(t);
   return cudaGetLastError();
 }
 
@@ -881,9 +1049,11 @@ cudaError_t launch_prune_trace(const DenseArgs& a, int32_t* guess, size_t guess_
   t.guess = guess;
   t.guess_cap = (int64_t)(guess_bytes / sizeof(int32_t));
   t.hdr = a.hdr;
-  if (a.K <= 256) return launch_trace_cfg<8>(t, max_T, st);
-  if (a.K <= 512) return launch_trace_cfg<16>(t, max_T, st);
-  return launch_trace_cfg<32>(t, max_T, st);
+  if (a.K <= 256) return launch_trace_cfg<8, 1>(t, max_T, st);
+  if (a.K <= 512) return launch_trace_cfg<16, 1>(t, max_T, st);
+  if (a.K <= 1024) return launch_trace_cfg<16, 2>(t, max_T, st);
+  if (a.K <= 2048) return launch_trace_cfg<16, 4>(t, max_T, st);
+  return launch_trace_cfg<16, 8>(t, max_T, st);
 }
 
 }  // namespace fv

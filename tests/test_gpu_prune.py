@@ -1,4 +1,4 @@
-"""The bounded-row engine (exact decoding, 128 < K <= 1024): paths and scores
+"""The bounded-row engine (exact decoding, 128 < K <= 4096): paths and scores
 against the oracle, bit for bit, at the edges of its tiles, launch
 configurations and trace segments, and on inputs that bound badly."""
 import numpy as np
@@ -53,6 +53,14 @@ def test_tile_and_segment_edges(fv, K):
     check(fv, log_pi, logA, [W.gaussian_emissions(t, K, rng) for t in T], pad=K % 3)
 
 
+@pytest.mark.parametrize("K,T", [(1025, [1, 49, 73, 90]), (1500, [2, 50, 97]), (2048, [48, 75]), (2049, [1, 51, 74]),
+                                 (3000, [60]), (4095, [49]), (4096, [50, 2])])
+def test_large_state_spaces(fv, K, T):
+    rng = np.random.default_rng(K)
+    log_pi, logA = W.random_model(K, rng, alpha=0.1 if K % 2 else 1.0)
+    check(fv, log_pi, logA, [W.gaussian_emissions(t, K, rng) for t in T], pad=K % 3)
+
+
 # launch configurations: jobs per SM and steps against the longest sequence
 @pytest.mark.parametrize("K,n,T", [(256, 1300, 40), (200, 700, 33), (300, 119, 30), (300, 121, 30), (512, 160, 25),
                                    (512, 400, 20), (700, 170, 20)])
@@ -64,7 +72,7 @@ def test_launch_configurations(fv, K, n, T):
     check(fv, log_pi, logA, E, sample=sorted(rng.choice(n, 24, replace=False)))
 
 
-@pytest.mark.parametrize("K", [144, 300, 600])
+@pytest.mark.parametrize("K", [144, 300, 600, 1100])
 @pytest.mark.parametrize("kind", ["flat", "spikes", "ties", "sparse", "constant", "negzero", "wide"])
 def test_inputs_that_bound_badly(fv, K, kind):
     rng = np.random.default_rng(K)
