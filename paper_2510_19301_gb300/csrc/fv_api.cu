@@ -251,10 +251,11 @@ int32_t beam_wcap(const fv_model* models, int32_t n_models, int32_t B) {
   return std::min(std::max(B, 1), kmax);
 }
 
-// Exact decoding keeps delta rows (T x K floats) instead of psi rows when
-// every model of the batch runs the bounded-row engine.
-bool delta_rows(const fv_model* models, int32_t n_models, int mode) {
-  if (mode != FV_VANILLA) return false;
+// Exact decoding keeps delta rows (T x K floats) instead of psi rows, and
+// the dynamic beam (P = 0) its entries' scores instead of their source
+// slots, when every model of the batch runs the bounded-row engine.
+bool delta_rows(const fv_model* models, int32_t n_models, const fv_params* p) {
+  if (p->mode != FV_VANILLA && !(p->mode == FV_BEAM && p->P < 1 && !(p->flags & FV_STATIC_BEAM))) return false;
   for (int m = 0; m < n_models; ++m)
     if (models[m].trans != FV_TRANS_DENSE || !dense_prune_K(models[m].K)) return false;
   return true;
@@ -292,12 +293,13 @@ Layout layout_for(const fv_model* models, int32_t n_models, const fv_batch* b, i
   }
   L.aux_elems = aux;
   size_t end = align_up(L.aux + aux * (mode == FV_VANILLA && !rows32 ? 2 : 4));
-  if (rows32) {
+  const bool table32 = rows32 && mode == FV_VANILLA;
+  if (table32) {
     size_t area = 0;
     for (int m = 0; m < n_models; ++m) area = std::max(area, prune_area_bytes(models[m].K));
     L.prune = end;
     L.guess = align_up(area);  // from L.prune
-    L.guess_bytes = prune_guess_bytes(aux, n, sum_T);
+    L.guess_bytes = prune_guess_bytes(aux, n, sum_T, 128);
     L.total = align_up(end + L.guess + L.guess_bytes);
     return L;
   }
@@ -388,6 +390,15 @@ Layout layout_for(const fv_model* models, int32_t n_models, const fv_batch* b, i
       end = align_up(L.div_n + 4 * (size_t)L.pe_cap * n);
     }
   }
+  if (rows32) {
+    // beam: the same areas behind the general engine's scratch
+    size_t area = 0;
+    for (int m = 0; m < n_models; ++m) area = std::max(area, prune_area_bytes(models[m].K));
+    L.prune = align_up(end);
+    L.guess = align_up(area);
+    L.guess_bytes = prune_guess_bytes(aux, n, sum_T, L.Wcap);
+    end = align_up(L.prune + L.guess + L.guess_bytes);
+  }
   L.total = end < 4096 ? 4096 : end;
   return L;
 }
@@ -453,7 +464,7 @@ void timed_end(cudaStream_t st) {
 // Beam search (P = 0) and FLASH-BS (P >= 1) launch sequence, per model.
 fv_status decode_beam(const fv_model* models, int32_t n_models, const fv_batch* batch, const fv_params* p, char* ws,
                       const Layout& L, const FlashPlan& fp, const Ranges& R, int32_t* paths_out, float* scores_out,
-                      cudaStream_t st) {
+                      bool prune, cudaStream_t st) {
   WsHeader* hdr = reinterpret_cast<WsHeader*>(ws + L.hdr);
   Job* jobs = reinterpret_cast<Job*>(ws + L.jobs);
   int32_t* order = reinterpret_cast<int32_t*>(ws + L.order);
@@ -503,6 +514,39 @@ fv_status decode_beam(const fv_model* models, int32_t n_models, const fv_batch* 
       }
     }
     if (m > 0 && launch_reset(ba.pop, st) != cudaSuccess) return FV_ECUDA;
+    if (prune && prune_beam_wins(md.K, ba.sum_T, ba.max_T, !ba.per_cta)) {
+      DenseArgs da;
+      memset(&da, 0, sizeof(da));
+      da.K = md.K;
+      da.logA = md.logA;
+      da.log_pi = md.log_pi;
+      da.emit = md.emit;
+      da.V = md.V;
+      da.logB = md.logB;
+      da.E = batch->E;
+      da.obs = batch->obs;
+      da.jobs = jobs;
+      da.order = order;
+      da.order_begin = R.begin[m];
+      da.order_count = R.count[m];
+      da.qlast = qlast;
+      da.scores = scores_out;
+      da.hdr = hdr;
+      da.beam_B = p->B;
+      da.beam_stride = L.Wcap;
+      da.beam_id = reinterpret_cast<int32_t*>(ws + L.aux);
+      da.beam_val = reinterpret_cast<float*>(ws + L.aux2);
+      int64_t all_T = 0;
+      for (int i = 0; i < batch->n_seq; ++i) all_T += batch->T_host[i];
+      if (launch_prune_prep(md.logA, md.K, ws + L.prune, &da, st) != cudaSuccess) return FV_ECUDA;
+      timed_begin(st);
+      if (launch_prune_beam(da, !ba.per_cta, st) != cudaSuccess) return FV_ECUDA;
+      timed_end(st);
+      if (launch_prune_trace(da, reinterpret_cast<int32_t*>(ws + L.prune + L.guess), L.guess_bytes, all_T,
+                             std::max(ba.max_T, 1), paths_out, st) != cudaSuccess)
+        return FV_ECUDA;
+      continue;
+    }
     if (!tasks) {
       ba.kind = kJobBeam;
       ba.bp_id = reinterpret_cast<int32_t*>(ws + L.aux);
@@ -629,8 +673,8 @@ size_t fv_workspace_size(const fv_model* models, int32_t n_models, const fv_batc
   if (p->mode == FV_BEAM && p->B < 1) return 0;
   if (p->mode != FV_VANILLA && p->mode != FV_BEAM && p->mode != FV_CHECKPOINT) return 0;
   const size_t base = layout_for(models, n_models, batch, p->mode, nullptr, p->B, p->P).total;
-  if (!delta_rows(models, n_models, p->mode)) return base;
-  return std::max(base, layout_for(models, n_models, batch, p->mode, nullptr, 0, 0, true).total);
+  if (!delta_rows(models, n_models, p)) return base;
+  return std::max(base, layout_for(models, n_models, batch, p->mode, nullptr, p->B, 0, true).total);
 }
 
 }  // extern "C"
@@ -672,11 +716,12 @@ fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* ba
   Layout L = layout_for(models, n_models, batch, p->mode, tasks ? &fp : nullptr, p->B, p->P);
   // exact decoding by the bounded-row engine, where the workspace holds the
   // delta rows (a workspace of the smaller, psi-row size keeps the others)
-  bool prune = batch->T_host && n > 0 && delta_rows(models, n_models, p->mode);
+  bool prune = batch->T_host && n > 0 && delta_rows(models, n_models, p);
   for (int m = 0; m < n_models && prune; ++m)
-    prune = dense_uses_prune(models[m].K, (p->flags & FV_NO_TUNE) != 0, (p->flags & FV_TEST_WITHHOLD_STEP) != 0);
+    prune = p->mode == FV_BEAM ||
+            dense_uses_prune(models[m].K, (p->flags & FV_NO_TUNE) != 0, (p->flags & FV_TEST_WITHHOLD_STEP) != 0);
   if (prune) {
-    const Layout LP = layout_for(models, n_models, batch, p->mode, nullptr, 0, 0, true);
+    const Layout LP = layout_for(models, n_models, batch, p->mode, nullptr, p->B, 0, true);
     prune = ws_bytes >= LP.total;
     if (prune) {
       // the copies go to the end of the workspace: whatever lies between is
@@ -688,7 +733,7 @@ fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* ba
   }
   if (batch->T_host && ws_bytes < L.total) return FV_ENOMEM;
   if (ws_bytes < L.aux) return FV_ENOMEM;
-  const uint64_t cap = prune ? (L.prune - L.aux) / 4 : (ws_bytes - L.aux) / (p->mode == FV_VANILLA ? 2 : 4);
+  const uint64_t cap = prune && p->mode == FV_VANILLA ? (L.prune - L.aux) / 4 : (ws_bytes - L.aux) / (p->mode == FV_VANILLA ? 2 : 4);
   if (n == 0) return FV_OK;
 
   char* ws = static_cast<char*>(workspace);
@@ -721,7 +766,7 @@ fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* ba
       if (launch_check_inputs(models[m], m, jobs, n, batch->E, batch->obs, hdr, st) != cudaSuccess) return FV_ECUDA;
   if (launch_order(jobs, n, (p->flags & FV_NO_SORT) ? 1 : 0, order, st) != cudaSuccess) return FV_ECUDA;
 
-  if (p->mode == FV_BEAM) return decode_beam(models, n_models, batch, p, ws, L, fp, R, paths_out, scores_out, st);
+  if (p->mode == FV_BEAM) return decode_beam(models, n_models, batch, p, ws, L, fp, R, paths_out, scores_out, prune, st);
 
   for (int m = 0; m < n_models; ++m) {
     if (!R.count[m]) continue;

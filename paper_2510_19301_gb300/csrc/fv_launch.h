@@ -133,6 +133,12 @@ struct DenseArgs {
   const uint16_t* pr_row;
   const float* pr_cut;
   float* pr_D;                // delta rows, T x K floats per sequence at job.aux_off
+  // dynamic beams on that engine: width (0: every state), entries per step
+  // of the table, states and scores of the entries at job.aux_off
+  int32_t beam_B;
+  int32_t beam_stride;
+  int32_t* beam_id;
+  float* beam_val;
   int32_t no_tune;            // use the default engine configuration, not the tuned one
   WsHeader* hdr;
 };
@@ -238,9 +244,11 @@ cudaError_t launch_small_forward(const DenseArgs& a, cudaStream_t st);
 size_t prune_area_bytes(int K);
 cudaError_t launch_prune_prep(const float* logA, int K, char* area, DenseArgs* a, cudaStream_t st);
 cudaError_t launch_prune_forward(const DenseArgs& a, int64_t sum_T, int max_T, cudaStream_t st);
-size_t prune_guess_bytes(uint64_t aux_elems, int32_t n_seq, int64_t sum_T);
+size_t prune_guess_bytes(uint64_t aux_elems, int32_t n_seq, int64_t sum_T, int32_t unit);
 cudaError_t launch_prune_trace(const DenseArgs& a, int32_t* guess, size_t guess_bytes, int64_t sum_T, int max_T,
                                int32_t* paths, cudaStream_t st);
+bool prune_beam_wins(int K, int64_t sum_T, int max_T, bool alone);
+cudaError_t launch_prune_beam(const DenseArgs& a, bool alone, cudaStream_t st);
 bool dense_prune_K(int K);
 bool dense_uses_prune(int K, bool no_tune, bool withhold);
 // AT[j * KD + i] = logA[i * K + j] (rows K..KD-1 are -inf), KD = wide_lane_stride(K).

@@ -184,8 +184,10 @@ constexpr float kGap = 0.85f, kGapCommon = 0.9f, kFarGap = 1.3f;
 // C = adjacent columns per lane (a job takes W = KP / (32 CL C) warps of each
 // CTA), G = jobs side by side, RES = the CTA's columns of logA are resident
 // in shared memory (else rows are read through L1 / L2), M = column list
-// length.
-template <int KP, int CL, int C, int G, bool RES, int M>
+// length, BEAM: a dynamic beam (Sec. V-C) instead of every state: delta is
+// -inf outside the beam, the top-B of the candidates is taken at the start of
+// the next step.
+template <int KP, int CL, int C, int G, bool RES, int M, bool BEAM>
 struct PruneCfg {
   static constexpr int KH = KP / CL, W = KH / (32 * C), NT = G * W * 32, NW = KP / 32;
   static constexpr int WB = NW < 8 ? NW : 8;  // words (of 32 rows) per list batch
@@ -197,7 +199,7 @@ struct PruneCfg {
   static constexpr size_t l_bytes = (size_t)G * W * CAP * 8;
   // COOP: the warps of a job build the first row list together, and a second
   // one of the rows the later pass is likely to want
-  static constexpr bool COOP = W > 1 && NW > 8;
+  static constexpr bool COOP = W > 1 && (NW > 8 || BEAM);
   static constexpr int NL = KP + U;  // entries of a common list
   static constexpr size_t s_bytes = COOP ? (size_t)G * 2 * NL * 8 : 0;
   static constexpr size_t smem = a_bytes + d_bytes + l_bytes + s_bytes;
@@ -205,9 +207,9 @@ struct PruneCfg {
 // bounded wait of the cluster exchange (~1 s at 2 GHz)
 constexpr long long kPruneWaitCycles = 1ll << 31;
 
-template <int KP, int CL, int C, int G, bool RES, int M>
-__global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_fwd_kernel(DenseArgs a) {
-  using Cfg = PruneCfg<KP, CL, C, G, RES, M>;
+template <int KP, int CL, int C, int G, bool RES, int M, bool BEAM>
+__global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M, BEAM>::NT, 1) prune_fwd_kernel(DenseArgs a) {
+  using Cfg = PruneCfg<KP, CL, C, G, RES, M, BEAM>;
   constexpr int KH = Cfg::KH, W = Cfg::W, NT = Cfg::NT, NW = Cfg::NW, CAP = Cfg::CAP, WB = Cfg::WB, U = Cfg::U;
   constexpr bool COOP = Cfg::COOP;
   extern __shared__ __align__(16) char smem[];
@@ -216,6 +218,13 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
   __shared__ uint32_t s_stop[CL];
   __shared__ float s_max[G][W], s_need[G][2][W];  // COOP: per warp maxima and depths
   __shared__ int s_cnt[G][2][2];                  // COOP: entries of the common lists, by step parity
+  // BEAM: candidates per bin (by step parity), those of the bin that holds
+  // the B-th, winners per warp
+  static_assert(!BEAM || (Cfg::COOP && G == 1), "beams: one job per CTA or cluster");
+  constexpr int BT = BEAM ? 128 : 1;
+  __shared__ __align__(16) int s_hist[BEAM ? 2 : 1][BEAM ? 256 : 4];
+  __shared__ float2 s_tie[BT];
+  __shared__ int s_ntie[2], s_win[W];
   const bool stop = a.hdr->status != 0;  // an earlier kernel recorded an error
   if (CL == 1 && stop) return;
   const int K = a.K;
@@ -295,7 +304,7 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
   const int ncl = (int)gridDim.x / CL, slots = ncl * G;
   const int cid = (int)blockIdx.x / CL;
   const int slot = grp * ncl + ((grp & 1) ? ncl - 1 - cid : cid);
-  bool live = true;
+  bool live = true, dead = false;
   uint32_t ph = 0;  // steps run so far: buffer ph & 1, its (ph >> 1)-th use
 
   for (int round = 0;; ++round) {
@@ -339,6 +348,12 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
       for (int c = 0; c < C; ++c) er[k][c] = 0.f;
       load_e(k, er[k]);
     }
+    float bref = 0.f, bscale = 32.f, bdepth = 4.f, binc = 0.f, bmax = 0.f;  // BEAM: bins of the top-B select
+    if constexpr (BEAM) {
+      for (int x = gt; x < 512; x += W * 32) s_hist[x >> 8][x & 255] = 0;
+      if (gt < 2) s_ntie[gt] = 0;
+      // (ordered by the barriers of the first step)
+    }
     float gap = 0.f;  // how far below the maximum this warp's last steps had to look
     for (int t = 0; t < T; ++t, ++ph) {
       const uint32_t cur = ph & 1u;  // buffer written by this step; cur ^ 1 is read
@@ -358,7 +373,7 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
         for (int c = 0; c < C; ++c)
           dval[c] = col0 + c < K ? __fadd_rn(__ldg(a.log_pi + col0 + c), e[c]) : -CUDART_INF_F;
       } else {
-        constexpr bool KEEP = NW <= 8;          // the deltas of this lane stay in registers
+        constexpr bool KEEP = NW <= 8 && !COOP;  // the deltas of this lane stay in registers
         constexpr int NK = COOP ? NW / W : NW;  // words this warp looks over for the maximum
         float dk[COOP && NK > WB ? NK : WB], dmax = -CUDART_INF_F;
 #pragma unroll
@@ -371,6 +386,179 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
         float lo, lo1 = 0.f;  // pass 0 takes delta >= lo; the second common list lo1 <= delta < lo
         int n = 0, n1 = 0;
         if constexpr (COOP) {
+          int win = 0;  // BEAM: winners of the lower lanes' rows in this warp, then this lane's
+          if constexpr (BEAM) {
+            // ---- top-B of the K candidates under (score desc, id asc).  A
+            // bin is a monotone function of the score, so whole bins above
+            // the B-th candidate's are taken and only that bin is ranked.
+            if (t == 1) {
+              if (lane == 0) s_max[grp][gw] = dmax;
+              group_any(false);
+#pragma unroll
+              for (int w = 0; w < W; ++w) dmax = fmaxf(dmax, s_max[grp][w]);
+              bref = bmax = dmax > -CUDART_INF_F ? dmax : 0.f;
+              group_any(false);
+            }
+            const int Wb = a.beam_B < K ? a.beam_B : K;
+            bool take[NK], in[NK];  // winners; candidates still to be decided
+#pragma unroll
+            for (int k = 0; k < NK; ++k) {
+              take[k] = false;
+              in[k] = dk[k] > -CUDART_INF_F;
+            }
+            // the bin that holds the B-th candidate, the winners in it, its size
+            int bb = 256, left = Wb, inb = 0, bb0 = 256;
+            bool open = false;
+#pragma unroll 1
+            for (int shift = 32;; shift -= 8) {
+              // bins of the score first; where more candidates share the bin
+              // than can be ranked (a wrong guess of the scale, or ties),
+              // radix passes over the ordered keys of those
+              int bin[NK];
+#pragma unroll
+              for (int k = 0; k < NK; ++k) {
+                if (shift == 32) {
+                  const float x = __fadd_rn(bref, -dk[k]) * bscale;
+                  bin[k] = x > 0.f ? (x < 255.f ? (int)x : 255) : 0;
+                } else {
+                  bin[k] = 255 - (int)((ord_key(__fadd_rn(dk[k], 0.f)) >> shift) & 0xffu);
+                }
+                if (in[k]) atomicAdd(&s_hist[cur][bin[k]], 1);
+              }
+              group_any(false);
+              const int4 h0 = *reinterpret_cast<const int4*>(&s_hist[cur][8 * lane]);
+              const int4 h1 = *reinterpret_cast<const int4*>(&s_hist[cur][8 * lane + 4]);
+              const int h[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+              int sum = 0;
+#pragma unroll
+              for (int x = 0; x < 8; ++x) sum += h[x];
+              int incl = sum;
+#pragma unroll
+              for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+              }
+              const int total = __shfl_sync(0xffffffffu, incl, 31);
+              bb = 256;
+              if (total > left) {
+                const int need = left;
+                int acc = incl - sum;
+#pragma unroll
+                for (int x = 0; x < 8; ++x) {
+                  if (acc < need && need <= acc + h[x]) {
+                    bb = 8 * lane + x;
+                    left = need - acc;
+                    inb = h[x];
+                  }
+                  acc += h[x];
+                }
+                const int src = __ffs(__ballot_sync(0xffffffffu, bb < 256)) - 1;
+                bb = __shfl_sync(0xffffffffu, bb, src);
+                left = __shfl_sync(0xffffffffu, left, src);
+                inb = __shfl_sync(0xffffffffu, inb, src);
+              } else if (total == 0) {
+                dead = true;  // the beam emptied: no finite path (every CTA sees the same)
+                break;
+              }
+              if (shift == 32) bb0 = bb;
+              open = bb < 256 && left < inb;
+#pragma unroll
+              for (int k = 0; k < NK; ++k) {
+                take[k] = take[k] || (in[k] && (bin[k] < bb || (bin[k] == bb && !open)));
+                in[k] = in[k] && open && bin[k] == bb;
+              }
+              if (!open || inb <= BT || shift == 0) break;
+              group_any(false);  // (the counts have been read)
+              for (int x = gt; x < 256; x += W * 32) s_hist[cur][x] = 0;
+              group_any(false);
+            }
+            if (dead) {
+              if (rank == 0 && gt == 0) set_status(a.hdr, FV_EINFEASIBLE, (uint32_t)b);
+              break;
+            }
+            for (int x = gt; x < 256; x += W * 32) s_hist[cur ^ 1u][x] = 0;
+            if (gt == 0) s_ntie[cur ^ 1u] = 0;
+            if (open && inb <= BT) {
+#pragma unroll
+              for (int k = 0; k < NK; ++k)
+                if (in[k])
+                  s_tie[atomicAdd(&s_ntie[cur], 1)] = make_float2(dk[k], __int_as_float(32 * (gw * NK + k) + lane));
+              group_any(false);
+              if (inb <= 32) {
+                // a lane per candidate: the last winner among them, for all
+                const float2 q = lane < inb ? s_tie[lane] : make_float2(-CUDART_INF_F, __int_as_float(0x7fffffff));
+                const int qi = __float_as_int(q.y);
+                int ahead = 0;
+                for (int x = 0; x < inb; ++x) {
+                  const float y = __shfl_sync(0xffffffffu, q.x, x);
+                  const int yi = __shfl_sync(0xffffffffu, qi, x);
+                  ahead += y > q.x || (y == q.x && yi < qi);
+                }
+                const int src = __ffs(__ballot_sync(0xffffffffu, lane < inb && ahead == left - 1)) - 1;
+                const float tv = __shfl_sync(0xffffffffu, q.x, src & 31);
+                const int ti = __shfl_sync(0xffffffffu, qi, src & 31);
+#pragma unroll
+                for (int k = 0; k < NK; ++k)
+                  if (in[k]) take[k] = dk[k] > tv || (dk[k] == tv && 32 * (gw * NK + k) + lane <= ti);
+              } else
+#pragma unroll
+              for (int k = 0; k < NK; ++k)
+                if (in[k]) {
+                  const int id = 32 * (gw * NK + k) + lane;
+                  int ahead = 0;
+                  for (int x = 0; x < inb; ++x) {
+                    const float2 q = s_tie[x];
+                    ahead += q.x > dk[k] || (q.x == dk[k] && __float_as_int(q.y) < id);
+                  }
+                  take[k] = ahead < left;
+                }
+            } else if (open) {
+              // more equal scores than the list holds: the lowest ids of them
+              int mine = 0;
+#pragma unroll
+              for (int k = 0; k < NK; ++k) mine += __popc(__ballot_sync(0xffffffffu, in[k]));
+              if (lane == 0) s_win[gw] = mine;
+              group_any(false);
+              int ahead = 0;
+#pragma unroll
+              for (int w = 0; w < W; ++w) ahead += w < gw ? s_win[w] : 0;
+#pragma unroll
+              for (int k = 0; k < NK; ++k) {
+                const uint32_t mk = __ballot_sync(0xffffffffu, in[k]);
+                if (in[k]) take[k] = ahead + __popc(mk & lt) < left;
+                ahead += __popc(mk);
+              }
+              group_any(false);  // (s_win is written again below)
+            }
+            // outside the beam: -inf, here and in the vector that is read
+            float* dm = sd + (cur ^ 1u) * KP;
+            dmax = -CUDART_INF_F;
+            int mine = 0;
+#pragma unroll
+            for (int k = 0; k < NK; ++k) {
+              if (!take[k]) {
+                if (dk[k] > -CUDART_INF_F) dm[32 * (gw * NK + k) + lane] = -CUDART_INF_F;
+                dk[k] = -CUDART_INF_F;
+              }
+              dmax = fmaxf(dmax, dk[k]);
+              mine += take[k];
+            }
+            dmax = warp_max_f32(dmax);
+            int x = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              const int y = __shfl_up_sync(0xffffffffu, x, o);
+              if (lane >= o) x += y;
+            }
+            win = x - mine;
+            if (lane == 31) s_win[gw] = x;
+            // the next step's bins: the B-th candidate near the middle
+            if (bb0 < 256) {
+              if (bb0 == 255) bdepth *= 1.5f;
+              else bdepth = 0.75f * bdepth + 0.25f * (((float)bb0 + 0.5f) / bscale);
+              bdepth = fmaxf(bdepth, fmaxf(0.25f * gap, 1e-30f));
+            }
+          }
           if (lane == 0) s_max[grp][gw] = dmax;
           if (gt < 2) s_cnt[grp][cur][gt] = 0;
           group_any(false);
@@ -380,6 +568,35 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
             dmax = fmaxf(dmax, s_max[grp][w]);
             const float x = s_need[grp][cur ^ 1u][w];
             most = fmaxf(most, x);
+          }
+          if constexpr (BEAM) {
+            // this CTA's winners of step t - 1 to the table (any order)
+            int pos = win, all = 0;
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+              const int x = s_win[w];
+              all += x;
+              if (w < gw) pos += x;
+            }
+            const int64_t base = jb.aux_off + (int64_t)(t - 1) * a.beam_stride;
+#pragma unroll
+            for (int k = 0; k < NK; ++k)
+              if (dk[k] > -CUDART_INF_F) {
+                const int id = 32 * (gw * NK + k) + lane;
+                if (CL == 1 || (id >= (int)rank * KH && id < ((int)rank + 1) * KH)) {
+                  a.beam_id[base + pos] = id;
+                  a.beam_val[base + pos] = dk[k];
+                }
+                ++pos;
+              }
+            for (int x = all + gt; x < a.beam_stride && rank == 0; x += W * 32) a.beam_id[base + x] = -1;
+            const float g = __fadd_rn(dmax, -bmax);
+            if (fabsf(g) < 1e30f) {
+              binc = 0.9f * binc + 0.1f * g;
+              bmax = dmax;
+            }
+            bref = __fadd_rn(bmax, binc);
+            bscale = 160.f / bdepth;
           }
           if (most >= 0.f) gap = 0.75f * gap + 0.25f * most;
           lo = fmaxf(__fmaf_rn(-kGapCommon, gap, dmax), -FLT_MAX);  // (never rows at -inf)
@@ -615,7 +832,9 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
           }
         }
       }
-      if (C > 1 && K % C == 0) {
+      if constexpr (BEAM) {
+        // (the beam of this step goes to the table once it is known)
+      } else if (C > 1 && K % C == 0) {
         if (col0 < K) {
           if constexpr (C == 4) __stcs(reinterpret_cast<float4*>(dt), make_float4(dval[0], dval[1], dval[2], dval[3]));
           if constexpr (C == 2) __stcs(reinterpret_cast<float2*>(dt), make_float2(dval[0], dval[1]));
@@ -648,6 +867,7 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
       }
     }
     if (!live) break;
+    if (BEAM && dead) break;
     if (rank == 0 && gw == 0) {
       // termination: q_{T-1} = lowest argmax_j delta_{T-1}[j], score = delta_{T-1}[q]
       const float* dl = sd + ((ph - 1u) & 1u) * KP;
@@ -665,10 +885,12 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
         if (ov > v || (ov == v && oq < qi)) { v = ov; qi = oq; }
       }
       if (lane == 0) {
+        if (BEAM && !(v > -CUDART_INF_F)) set_status(a.hdr, FV_EINFEASIBLE, (uint32_t)b);
         a.qlast[b] = qi;
         a.scores[b] = dl[qi];
       }
     }
+    if constexpr (BEAM && CL == 1) group_any(false);  // (the next job clears what this one read)
   }
   if constexpr (CL > 1) {
     // no CTA leaves while another may still write to it or read its barriers
@@ -689,35 +911,65 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M>::NT, 1) prune_f
 // the path's state until it meets the written path.
 constexpr int kTraceWarm = 24;
 
+struct TraceArgs {
+  const Job* jobs;
+  const int32_t* order;
+  int32_t begin, count, K, seg;  // seg: states per segment
+  int32_t row, unit;             // BEAM: entries per row; at most this many table elements per step
+  const int32_t* ids;            // BEAM: states of the entries
+  const float* D;
+  const float* AT;
+  const int32_t* qlast;
+  int32_t* paths;
+  int32_t* guess;  // state assumed at each segment's end
+  int64_t guess_cap;
+  const WsHeader* hdr;
+};
 // TW warps of a CTA follow one chain, VPL rows of a column per thread.
-template <int VPL, int TW>
+template <int VPL, int TW, bool BEAM>
 struct Tracer {
   static constexpr int AH = VPL <= 8 ? 4 : 2;  // delta rows loaded ahead
   static constexpr int NT = 32 * TW;
-  const float* D;
+  const float* D;     // delta rows, or the beams' scores
+  const int32_t* ids;  // BEAM: their states (-1: no entry)
   const float* AT;
   int K, KD, tid;
+  int N;  // entries of a row
   uint2* part;  // shared, [2][TW]: per warp (value, row) of a step, by turns
   int turn;
-  float d[AH][VPL];
-  __device__ __forceinline__ void init(const float* D_, const float* AT_, int K_, uint2* part_) {
-    D = D_;
-    AT = AT_;
+  struct Row {
+    float d[VPL];
+    int i[BEAM ? VPL : 1];
+  };
+  Row rows[AH];
+  __device__ __forceinline__ void init(const TraceArgs& a, const Job& jb, uint2* part_) {
+    D = a.D + jb.aux_off;
+    if (BEAM) ids = a.ids + jb.aux_off;
+    AT = a.AT;
+    N = BEAM ? a.row : a.K;
+    const int K_ = a.K;
     K = K_;
     KD = wide_lane_stride(K_);
     tid = threadIdx.x;
     part = part_;
     turn = 0;
   }
-  __device__ __forceinline__ void load(int t, float (&x)[VPL]) {
+  __device__ __forceinline__ void load(int t, Row& x) {
 #pragma unroll
-    for (int k = 0; k < VPL; ++k)
-      x[k] = (t >= 0 && NT * k + tid < K) ? __ldcs(D + (int64_t)t * K + NT * k + tid) : -CUDART_INF_F;
+    for (int k = 0; k < VPL; ++k) {
+      const int e = NT * k + tid;
+      const bool in = t >= 0 && e < N;
+      if constexpr (BEAM) {
+        x.i[k] = in ? __ldcs(ids + (int64_t)t * N + e) : -1;
+        if ((unsigned)x.i[k] >= (unsigned)K) x.i[k] = -1;
+      }
+      x.d[k] = in ? __ldcs(D + (int64_t)t * N + e) : -CUDART_INF_F;
+    }
   }
   // rows t - 1, t - 2, ... for steps from state q_t downwards
   __device__ __forceinline__ void start(int t) {
 #pragma unroll
-    for (int k = 0; k < AH; ++k) load(t - 1 - k, d[k]);
+    for (int k = 0; k < AH; ++k) load(t - 1 - k, rows[k]);
   }
   // lowest argmax over the threads' (value, row); 0 where every value is -inf
   __device__ __forceinline__ int lowest(float bv, int bi) {
@@ -741,30 +993,38 @@ struct Tracer {
     return r < (uint32_t)K ? (int)r : 0;
   }
   // q_{t-1} from q_t; `x` holds delta_{t-1} and receives row t - 1 - AH
-  __device__ __forceinline__ int step(int t, int q, float (&x)[VPL]) {
-    const float* col = AT + (int64_t)q * KD + tid;
+  __device__ __forceinline__ int step(int t, int q, Row& x) {
+    const float* col = AT + (int64_t)q * KD;
     float v[VPL];
 #pragma unroll
-    for (int k = 0; k < VPL; ++k) v[k] = NT * k + tid < KD ? __ldg(col + NT * k) : -CUDART_INF_F;
+    for (int k = 0; k < VPL; ++k) {
+      const int i = BEAM ? x.i[k] : NT * k + tid;
+      v[k] = (BEAM ? i >= 0 : i < KD) ? __ldg(col + i) : -CUDART_INF_F;
+    }
     float bv = -CUDART_INF_F;
     int bi = 0;
 #pragma unroll
-    for (int k = 0; k < VPL; ++k) {
-      const float c = __fadd_rn(x[k], v[k]);
-      if (c > bv) { bv = c; bi = NT * k + tid; }
-    }
+    for (int k = 0; k < VPL; ++k) pick(__fadd_rn(x.d[k], v[k]), x, k, bv, bi);
     load(t - 1 - AH, x);
     return lowest(bv, bi);
   }
+  // (value, row) of entry k, if it comes before (bv, bi)
+  __device__ __forceinline__ void pick(float c, const Row& x, int k, float& bv, int& bi) {
+    if constexpr (BEAM) {
+      // a row's entries come in any order
+      if (x.i[k] >= 0 && (c > bv || (c == bv && x.i[k] < bi))) { bv = c; bi = x.i[k]; }
+    } else {
+      if (c > bv) { bv = c; bi = NT * k + tid; }
+    }
+  }
   // lowest argmax of delta_t
   __device__ __forceinline__ int best(int t) {
-    float x[VPL];
+    Row x;
     load(t, x);
     float bv = -CUDART_INF_F;
     int bi = 0;
 #pragma unroll
-    for (int k = 0; k < VPL; ++k)
-      if (x[k] > bv) { bv = x[k]; bi = NT * k + tid; }
+    for (int k = 0; k < VPL; ++k) pick(x.d[k], x, k, bv, bi);
     return lowest(bv, bi);
   }
   // from q_t down to state `to`; f(time, state) returns true to stop there
@@ -775,7 +1035,7 @@ struct Tracer {
 #pragma unroll
       for (int s = 0; s < AH; ++s) {
         if (t <= to) break;
-        q = step(t, q, d[s]);
+        q = step(t, q, rows[s]);
         --t;
         if (f(t, q)) return q;
       }
@@ -784,24 +1044,13 @@ struct Tracer {
   }
 };
 
-struct TraceArgs {
-  const Job* jobs;
-  const int32_t* order;
-  int32_t begin, count, K, seg;  // seg: states per segment
-  const float* D;
-  const float* AT;
-  const int32_t* qlast;
-  int32_t* paths;
-  int32_t* guess;  // state assumed at each segment's end
-  int64_t guess_cap;
-  const WsHeader* hdr;
-};
-// first guess of a sequence (at least ceil(T / seg) apart, as K > 128)
+// first guess of a sequence: at least ceil(T / seg) apart, as a step has
+// `unit` table elements or more
 __device__ __forceinline__ int64_t guess_off(const TraceArgs& a, const Job& jb, int b) {
-  return jb.aux_off / (128ll * a.seg) + b;
+  return jb.aux_off / ((int64_t)a.unit * a.seg) + b;
 }
 
-template <int VPL, int TW>
+template <int VPL, int TW, bool BEAM>
 __global__ void __launch_bounds__(32 * TW) prune_trace_kernel(TraceArgs a) {
   __shared__ uint2 part[2 * TW];
   if (a.hdr->status != 0) return;
@@ -809,8 +1058,8 @@ __global__ void __launch_bounds__(32 * TW) prune_trace_kernel(TraceArgs a) {
   const Job jb = a.jobs[b];
   const int s = blockIdx.y, T = jb.T, K = a.K, lo = s * a.seg;
   if (lo >= T) return;
-  Tracer<VPL, TW> tr;
-  tr.init(a.D + jb.aux_off, a.AT, K, part);
+  Tracer<VPL, TW, BEAM> tr;
+  tr.init(a, jb, part);
   int32_t* path = a.paths + jb.path_off;
   const bool lead = threadIdx.x == 0;
   int q = a.qlast[b];
@@ -835,7 +1084,7 @@ __global__ void __launch_bounds__(32 * TW) prune_trace_kernel(TraceArgs a) {
   });
 }
 
-template <int VPL, int TW>
+template <int VPL, int TW, bool BEAM>
 __global__ void __launch_bounds__(32 * TW) prune_fix_kernel(TraceArgs a) {
   __shared__ uint2 part[2 * TW];
   if (a.hdr->status != 0) return;
@@ -860,8 +1109,8 @@ __global__ void __launch_bounds__(32 * TW) prune_fix_kernel(TraceArgs a) {
       continue;
     }
     const int sb = s1 - (__ffs(m) - 1), lo = sb * a.seg, hi = lo + a.seg;
-    Tracer<VPL, TW> tr;
-    tr.init(a.D + jb.aux_off, a.AT, K, part);
+    Tracer<VPL, TW, BEAM> tr;
+    tr.init(a, jb, part);
     int q = __ldcg(path + hi);
     q = (unsigned)q < (unsigned)K ? q : 0;
     sync();
@@ -925,12 +1174,12 @@ cudaError_t launch_prune_prep(const float* logA, int K, char* area, DenseArgs* a
 
 // Clusters (CTAs for CL = 1) of a configuration resident at once; 0 where the
 // device does not take it.
-template <int KP, int CL, int C, int G, bool RES, int M>
+template <int KP, int CL, int C, int G, bool RES, int M, bool BEAM>
 static int prune_resident(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
-  using Cfg = PruneCfg<KP, CL, C, G, RES, M>;
+  using Cfg = PruneCfg<KP, CL, C, G, RES, M, BEAM>;
   static_assert(Cfg::smem + 1024 <= 227 * 1024, "one CTA per SM");
   static_assert(Cfg::W == 1 || G <= 15, "a named barrier per job group");
-  auto kern = prune_fwd_kernel<KP, CL, C, G, RES, M>;
+  auto kern = prune_fwd_kernel<KP, CL, C, G, RES, M, BEAM>;
   int n = 0;
   const int nsm = device_sm_count();
   attr->id = cudaLaunchAttributeClusterDimension;
@@ -959,15 +1208,15 @@ static int prune_resident(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
   return n;
 }
 
-template <int KP, int CL, int C, int G, bool RES, int M>
+template <int KP, int CL, int C, int G, bool RES, int M, bool BEAM>
 static cudaError_t launch_prune_cfg(const DenseArgs& a, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
-  const int resident = prune_resident<KP, CL, C, G, RES, M>(&cfg, attr), jobs = a.order_count;
+  const int resident = prune_resident<KP, CL, C, G, RES, M, BEAM>(&cfg, attr), jobs = a.order_count;
   if (resident < 1) return cudaErrorInvalidConfiguration;
   cfg.stream = st;
   cfg.gridDim = dim3(CL * (jobs < resident ? jobs : resident));
-  return cudaLaunchKernelEx(&cfg, prune_fwd_kernel<KP, CL, C, G, RES, M>, a);
+  return cudaLaunchKernelEx(&cfg, prune_fwd_kernel<KP, CL, C, G, RES, M, BEAM>, a);
 }
 
 // Configurations by state count and launch (GB300, us per step of the whole
@@ -996,20 +1245,20 @@ cudaError_t launch_prune_forward(const DenseArgs& a, int64_t sum_T, int max_T, c
   const int jobs = a.order_count, nsm = device_sm_count();
   if (jobs <= 0) return cudaSuccess;
   if (a.K <= 256) {
-    if (sum_T > 5ll * nsm * max_T) return launch_prune_cfg<256, 2, 4, 16, true, 6>(a, st);
-    return launch_prune_cfg<256, 2, 2, 8, true, 6>(a, st);
+    if (sum_T > 5ll * nsm * max_T) return launch_prune_cfg<256, 2, 4, 16, true, 6, false>(a, st);
+    return launch_prune_cfg<256, 2, 2, 8, true, 6, false>(a, st);
   }
   if (a.K <= 512) {
-    if (jobs <= 120) return launch_prune_cfg<512, 8, 2, 8, true, 12>(a, st);
-    if (jobs <= nsm) return launch_prune_cfg<512, 1, 2, 1, false, 12>(a, st);
-    return launch_prune_cfg<512, 1, 4, 1, false, 12>(a, st);
+    if (jobs <= 120) return launch_prune_cfg<512, 8, 2, 8, true, 12, false>(a, st);
+    if (jobs <= nsm) return launch_prune_cfg<512, 1, 2, 1, false, 12, false>(a, st);
+    return launch_prune_cfg<512, 1, 4, 1, false, 12, false>(a, st);
   }
   if (a.K <= 1024) {
-    if (2 * jobs <= nsm) return launch_prune_cfg<1024, 2, 2, 1, false, 16>(a, st);
-    return launch_prune_cfg<1024, 1, 4, 1, false, 16>(a, st);
+    if (2 * jobs <= nsm) return launch_prune_cfg<1024, 2, 2, 1, false, 16, false>(a, st);
+    return launch_prune_cfg<1024, 1, 4, 1, false, 16, false>(a, st);
   }
-  if (a.K <= 2048) return launch_prune_cfg<2048, 4, 2, 1, false, 32>(a, st);
-  return launch_prune_cfg<4096, 8, 2, 1, false, 32>(a, st);
+  if (a.K <= 2048) return launch_prune_cfg<2048, 4, 2, 1, false, 32, false>(a, st);
+  return launch_prune_cfg<4096, 8, 2, 1, false, 32, false>(a, st);
 }
 
 // States per segment of the trace: a few thousand segments over the launch,
@@ -1018,21 +1267,34 @@ int prune_trace_seg(int64_t sum_T) {
   const int64_t s = (sum_T / 4096 + 15) / 16 * 16;
   return (int)(s < 48 ? 48 : s > 512 ? 512 : s);
 }
-size_t prune_guess_bytes(uint64_t aux_elems, int32_t n_seq, int64_t sum_T) {
-  return sizeof(int32_t) * (size_t)(aux_elems / (128ull * (uint64_t)prune_trace_seg(sum_T)) + (uint64_t)n_seq + 1ull);
+// `unit`: table elements per step at least (128 for delta rows, the beam
+// table's row length)
+size_t prune_guess_bytes(uint64_t aux_elems, int32_t n_seq, int64_t sum_T, int32_t unit) {
+  const uint64_t per = (uint64_t)unit * (uint64_t)prune_trace_seg(sum_T);
+  return sizeof(int32_t) * (size_t)(aux_elems / per + (uint64_t)n_seq + 1ull);
 }
 
-template <int VPL, int TW>
+template <int VPL, int TW, bool BEAM>
 static cudaError_t launch_trace_cfg(const TraceArgs& t, int max_T, cudaStream_t st) {
   const dim3 grid(t.count, (max_T + t.seg - 1) / t.seg);
-  prune_trace_kernel<VPL, TW><<<grid, 32 * TW, 0, st>>>(t);
-  if (grid.y > 1) prune_fix_kernel<VPL, TW><<<t.count, 32 * TW, 0, st>>>(t);
+  prune_trace_kernel<VPL, TW, BEAM><<<grid, 32 * TW, 0, st>>>(t);
+  if (grid.y > 1) prune_fix_kernel<VPL, TW, BEAM><<<t.count, 32 * TW, 0, st>>>(t);
   return cudaGetLastError();
+}
+
+template <bool BEAM>
+static cudaError_t launch_trace(const TraceArgs& t, int n, int max_T, cudaStream_t st) {
+  if (n <= 256) return launch_trace_cfg<8, 1, BEAM>(t, max_T, st);
+  if (n <= 512) return launch_trace_cfg<16, 1, BEAM>(t, max_T, st);
+  if (n <= 1024) return launch_trace_cfg<16, 2, BEAM>(t, max_T, st);
+  if (n <= 2048) return launch_trace_cfg<16, 4, BEAM>(t, max_T, st);
+  return launch_trace_cfg<16, 8, BEAM>(t, max_T, st);
 }
 
 cudaError_t launch_prune_trace(const DenseArgs& a, int32_t* guess, size_t guess_bytes, int64_t sum_T, int max_T,
                                int32_t* paths, cudaStream_t st) {
   if (a.order_count <= 0) return cudaSuccess;
+  const bool beam = a.beam_B > 0;
   TraceArgs t;
   t.jobs = a.jobs;
   t.order = a.order;
@@ -1042,18 +1304,47 @@ cudaError_t launch_prune_trace(const DenseArgs& a, int32_t* guess, size_t guess_
   t.seg = prune_trace_seg(sum_T);
   // (grid.y is at most 65535)
   if (max_T / t.seg > 32768) t.seg = (max_T / 32768 + 1) * t.seg;
-  t.D = a.pr_D;
+  t.row = a.beam_stride;
+  t.unit = beam ? a.beam_stride : 128;
+  t.ids = a.beam_id;
+  t.D = beam ? a.beam_val : a.pr_D;
   t.AT = a.wide_AT;
   t.qlast = a.qlast;
   t.paths = paths;
   t.guess = guess;
   t.guess_cap = (int64_t)(guess_bytes / sizeof(int32_t));
   t.hdr = a.hdr;
-  if (a.K <= 256) return launch_trace_cfg<8, 1>(t, max_T, st);
-  if (a.K <= 512) return launch_trace_cfg<16, 1>(t, max_T, st);
-  if (a.K <= 1024) return launch_trace_cfg<16, 2>(t, max_T, st);
-  if (a.K <= 2048) return launch_trace_cfg<16, 4>(t, max_T, st);
-  return launch_trace_cfg<16, 8>(t, max_T, st);
+  return beam ? launch_trace<true>(t, a.beam_stride, max_T, st) : launch_trace<false>(t, a.K, max_T, st);
+}
+
+// Dynamic beams (P = 0) over the same step; `alone`: the call has the GPU to
+// itself, so a launch may spread a sequence over more than one SM.
+// Measured against fv_beam.cu, us per step of the whole call (GB300): K = 256,
+// B = 64, 70 sequences 20.4 -> 2.9; K = 512, B = 128, 64 sequences 14.4 -> 4.8;
+// K = 1024, B = 256, 40 sequences 27.7 -> 8.7, one sequence 8.7 -> 6.5.  At 1024
+// < K <= 2048 a sequence takes a cluster of four CTAs (36 at a time; K = 2048,
+// B = 256, one sequence 12.0 -> 10.2, 64 sequences 34.7 -> 21.8), so the launch
+// is compared with one CTA per sequence on fv_beam.cu, whose step takes 3
+// times as long or more; K = 4096 was no faster (one sequence 17.8 -> 21.5).
+// Returns false where fv_beam.cu wins.
+bool prune_beam_wins(int K, int64_t sum_T, int max_T, bool alone) {
+  if (K <= 1024) return true;
+  if (!alone || K > 2048) return false;
+  const int64_t nsm = device_sm_count(), ncl = nsm / 4 - 2;
+  const int64_t here = max_T > sum_T / ncl ? max_T : sum_T / ncl, there = max_T > sum_T / nsm ? max_T : sum_T / nsm;
+  return here < 3 * there;
+}
+
+cudaError_t launch_prune_beam(const DenseArgs& a, bool alone, cudaStream_t st) {
+  const int jobs = a.order_count, nsm = device_sm_count();
+  if (jobs <= 0) return cudaSuccess;
+  if (a.K <= 256) return launch_prune_cfg<256, 1, 1, 1, false, 6, true>(a, st);
+  if (a.K <= 512) return launch_prune_cfg<512, 1, 2, 1, false, 12, true>(a, st);
+  if (a.K <= 1024) {
+    if (alone && 2 * jobs <= nsm) return launch_prune_cfg<1024, 2, 2, 1, false, 16, true>(a, st);
+    return launch_prune_cfg<1024, 1, 4, 1, false, 16, true>(a, st);
+  }
+  return launch_prune_cfg<2048, 4, 2, 1, false, 32, true>(a, st);
 }
 
 }  // namespace fv

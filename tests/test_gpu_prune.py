@@ -155,3 +155,69 @@ def test_small_workspace_keeps_the_backpointer_engines(fv, K):
     p0, s0 = (x.clone() for x in big())
     p1, s1 = small()
     assert torch.equal(p0, p1) and torch.equal(s0, s1)
+
+
+def check_beam(fv, log_pi, logA, E_list, B, flags=0):
+    K = log_pi.shape[0]
+    T = [e.shape[0] for e in E_list]
+    m = fv.Model(log_pi, logA)
+    b = fv.Batch(T, E=torch.from_numpy(np.concatenate(E_list)).cuda(), models=[m])
+    paths, scores = fv.decode([m], b, mode="beam", B=B, P=0, flags=flags)
+    paths, scores = paths.cpu().numpy(), scores.cpu().numpy()
+    hmm = oracle.HMM(log_pi, logA)
+    o = 0
+    for i, r in enumerate(oracle.map_sequences(lambda e: oracle.beam(hmm, e, B), E_list)):
+        assert r[-1] == 0
+        assert np.array_equal(paths[o:o + T[i]], r[0]), f"K={K} B={B} sequence {i} (T={T[i]}) path"
+        assert bits(scores[i]) == bits(r[1]), f"K={K} B={B} sequence {i} score"
+        o += T[i]
+
+
+# every padded size, one and several CTAs per sequence (the shared-GPU flag
+# keeps one at K <= 1024); 80 sequences: one CTA each
+@pytest.mark.parametrize("K,B,n,shared", [(129, 7, 4, 0), (256, 255, 4, 0), (257, 64, 4, 1), (512, 100, 4, 0), (513, 33, 4, 0),
+                                          (1024, 256, 4, 0), (1000, 200, 4, 1), (700, 90, 80, 0), (1025, 128, 3, 0),
+                                          (2048, 500, 2, 0)])
+def test_beam_sizes(fv, K, B, n, shared):
+    rng = np.random.default_rng(K + B)
+    log_pi, logA = W.random_model(K, rng)
+    T = [1, 2, 49, 80][:n] if n <= 4 else list(rng.integers(1, 30, n))
+    check_beam(fv, log_pi, logA, [W.gaussian_emissions(int(t), K, rng) for t in T], B,
+               flags=fv._lib.FV_SHARED_GPU if shared else 0)
+
+
+# the select: one bin holds more candidates than are ranked (equal scores,
+# one common value, scores of another scale from step to step), B = 1, B >= K
+@pytest.mark.parametrize("K", [150, 600, 1100])
+@pytest.mark.parametrize("kind,B", [("ties", 40), ("equal", 100), ("scale", 64), ("plain", 1), ("plain", 5000),
+                                    ("jump", 90)])
+def test_beam_select(fv, K, kind, B):
+    rng = np.random.default_rng(K + B)
+    log_pi, logA = W.random_model(K, rng)
+    T = [40, 1, 60]
+    E = [W.gaussian_emissions(t, K, rng) for t in T]
+    if kind == "ties":
+        logA = rng.integers(-2, 3, (K, K)).astype(np.float32)
+        log_pi = rng.integers(-2, 3, K).astype(np.float32)
+        E = [rng.integers(-1, 2, e.shape).astype(np.float32) for e in E]
+    elif kind == "equal":
+        logA[:] = -2.0
+        log_pi[:] = -0.0
+        E = [np.zeros_like(e) for e in E]
+    elif kind == "scale":
+        E = [(e * np.where(np.arange(len(e)) % 7 == 3, 1e4, 1e-3)[:, None]).astype(np.float32) for e in E]
+    elif kind == "jump":  # the common level of the scores moves by far more than their spread
+        E = [(e + np.where(np.arange(len(e)) % 5 == 2, 3e3, -8e2)[:, None]).astype(np.float32) for e in E]
+    check_beam(fv, log_pi, logA, E, B)
+
+
+@pytest.mark.parametrize("K", [200, 900])
+def test_beam_that_empties_is_reported(fv, K):
+    rng = np.random.default_rng(K)
+    log_pi, logA = W.random_model(K, rng)
+    logA[:, :] = -np.inf
+    m = fv.Model(log_pi, logA)
+    b = fv.Batch([20, 5], E=torch.from_numpy(W.gaussian_emissions(25, K, rng)).cuda(), models=[m])
+    d = fv.Decoder([m], b, mode="beam", B=16, P=0)
+    d.launch()
+    assert d.device_status() == fv._lib.FV_EINFEASIBLE
