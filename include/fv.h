@@ -57,8 +57,8 @@ typedef enum {
 
 typedef enum {
   FV_VANILLA = 0,   /* full table + backtrack (Sec. III-A): T x K uint16 backpointers,
-                       or T x K delta values (128 < K <= 4096, where the workspace
-                       has room: fv_workspace_size asks for them)               */
+                       or T x K delta values where the workspace has room
+                       (fv_workspace_size asks for them)                        */
   FV_FLASH = 1,     /* non-recursive D&C with MidState (Alg. 1, Alg. 2)            */
   FV_BEAM = 2,      /* dynamic beam (Sec. V-C); P >= 1 makes it FLASH-BS          */
   FV_CHECKPOINT = 3 /* Checkpoint Viterbi, the baseline of Sec. II-A (see below)  */

@@ -239,6 +239,7 @@ struct Layout {
   size_t at;         // column-major logA copy of the streamed configurations (256 < K <= 1024)
   size_t prune;      // bounded-row engine: copies and column lists of the largest model, then
   size_t guess, guess_bytes;  // the trace's segment ends
+  int32_t unit;               // table elements of a step at least
   uint64_t aux_elems;
   int64_t map_stride, snap_stride, list_cap;
   int32_t Wcap, Bcap, pe_cap, max_ctas;
@@ -257,7 +258,9 @@ int32_t beam_wcap(const fv_model* models, int32_t n_models, int32_t B) {
 bool delta_rows(const fv_model* models, int32_t n_models, const fv_params* p) {
   if (p->mode != FV_VANILLA && !(p->mode == FV_BEAM && p->P < 1 && !(p->flags & FV_STATIC_BEAM))) return false;
   for (int m = 0; m < n_models; ++m)
-    if (models[m].trans != FV_TRANS_DENSE || !dense_prune_K(models[m].K)) return false;
+    if (models[m].trans != FV_TRANS_DENSE || !dense_prune_K(models[m].K) ||
+        (p->mode == FV_BEAM && models[m].K <= 128))
+      return false;
   return true;
 }
 
@@ -299,7 +302,9 @@ Layout layout_for(const fv_model* models, int32_t n_models, const fv_batch* b, i
     for (int m = 0; m < n_models; ++m) area = std::max(area, prune_area_bytes(models[m].K));
     L.prune = end;
     L.guess = align_up(area);  // from L.prune
-    L.guess_bytes = prune_guess_bytes(aux, n, sum_T, 128);
+    L.unit = 128;
+    for (int m = 0; m < n_models; ++m) L.unit = std::min(L.unit, models[m].K);
+    L.guess_bytes = prune_guess_bytes(aux, n, sum_T, L.unit);
     L.total = align_up(end + L.guess + L.guess_bytes);
     return L;
   }
@@ -396,7 +401,8 @@ Layout layout_for(const fv_model* models, int32_t n_models, const fv_batch* b, i
     for (int m = 0; m < n_models; ++m) area = std::max(area, prune_area_bytes(models[m].K));
     L.prune = align_up(end);
     L.guess = align_up(area);
-    L.guess_bytes = prune_guess_bytes(aux, n, sum_T, L.Wcap);
+    L.unit = L.Wcap;
+    L.guess_bytes = prune_guess_bytes(aux, n, sum_T, L.unit);
     end = align_up(L.prune + L.guess + L.guess_bytes);
   }
   L.total = end < 4096 ? 4096 : end;
@@ -542,7 +548,7 @@ fv_status decode_beam(const fv_model* models, int32_t n_models, const fv_batch* 
       timed_begin(st);
       if (launch_prune_beam(da, !ba.per_cta, st) != cudaSuccess) return FV_ECUDA;
       timed_end(st);
-      if (launch_prune_trace(da, reinterpret_cast<int32_t*>(ws + L.prune + L.guess), L.guess_bytes, all_T,
+      if (launch_prune_trace(da, reinterpret_cast<int32_t*>(ws + L.prune + L.guess), L.guess_bytes, all_T, L.unit,
                              std::max(ba.max_T, 1), paths_out, st) != cudaSuccess)
         return FV_ECUDA;
       continue;
@@ -720,6 +726,14 @@ fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* ba
   for (int m = 0; m < n_models && prune; ++m)
     prune = p->mode == FV_BEAM ||
             dense_uses_prune(models[m].K, (p->flags & FV_NO_TUNE) != 0, (p->flags & FV_TEST_WITHHOLD_STEP) != 0);
+  // (preparing a model above K = 2048 costs more than the whole-GPU engine's
+  // steps up to about 30: K = 4096, 5 / 20 steps 326 / 497 against 210 / 482 us)
+  if (prune && p->mode == FV_VANILLA) {
+    int32_t kmax = 0, tmax = 0;
+    for (int m = 0; m < n_models; ++m) kmax = std::max(kmax, models[m].K);
+    for (int i = 0; i < n; ++i) tmax = std::max(tmax, batch->T_host[i]);
+    prune = kmax <= 2048 || tmax >= 32;
+  }
   if (prune) {
     const Layout LP = layout_for(models, n_models, batch, p->mode, nullptr, p->B, 0, true);
     prune = ws_bytes >= LP.total;
@@ -798,7 +812,7 @@ fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* ba
     if (prune) {
       da.kind = kJobVanilla;
       da.pr_D = reinterpret_cast<float*>(ws + L.aux);
-      if (launch_prune_prep(md.logA, md.K, ws + L.prune, &da, st) != cudaSuccess) return FV_ECUDA;
+      if (md.K > 128 && launch_prune_prep(md.logA, md.K, ws + L.prune, &da, st) != cudaSuccess) return FV_ECUDA;
       int64_t sum_T = 0, all_T = 0;
       int32_t max_T = 1;
       for (int i = 0; i < n; ++i) {
@@ -808,9 +822,10 @@ fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* ba
         max_T = std::max(max_T, batch->T_host[i]);
       }
       timed_begin(st);
-      if (launch_prune_forward(da, sum_T, max_T, st) != cudaSuccess) return FV_ECUDA;
+      if ((md.K <= 128 ? launch_small_values(da, st) : launch_prune_forward(da, sum_T, max_T, st)) != cudaSuccess)
+        return FV_ECUDA;
       timed_end(st);
-      if (launch_prune_trace(da, reinterpret_cast<int32_t*>(ws + L.prune + L.guess), L.guess_bytes, all_T, max_T,
+      if (launch_prune_trace(da, reinterpret_cast<int32_t*>(ws + L.prune + L.guess), L.guess_bytes, all_T, L.unit, max_T,
                              paths_out, st) != cudaSuccess)
         return FV_ECUDA;
       continue;

@@ -245,12 +245,14 @@ size_t prune_area_bytes(int K);
 cudaError_t launch_prune_prep(const float* logA, int K, char* area, DenseArgs* a, cudaStream_t st);
 cudaError_t launch_prune_forward(const DenseArgs& a, int64_t sum_T, int max_T, cudaStream_t st);
 size_t prune_guess_bytes(uint64_t aux_elems, int32_t n_seq, int64_t sum_T, int32_t unit);
-cudaError_t launch_prune_trace(const DenseArgs& a, int32_t* guess, size_t guess_bytes, int64_t sum_T, int max_T,
-                               int32_t* paths, cudaStream_t st);
+cudaError_t launch_prune_trace(const DenseArgs& a, int32_t* guess, size_t guess_bytes, int64_t sum_T, int unit,
+                               int max_T, int32_t* paths, cudaStream_t st);
 bool prune_beam_wins(int K, int64_t sum_T, int max_T, bool alone);
 cudaError_t launch_prune_beam(const DenseArgs& a, bool alone, cudaStream_t st);
 bool dense_prune_K(int K);
 bool dense_uses_prune(int K, bool no_tune, bool withhold);
+// exact decoding at K <= 128, values only: delta rows to a.pr_D (fv_small.cu)
+cudaError_t launch_small_values(const DenseArgs& a, cudaStream_t st);
 // AT[j * KD + i] = logA[i * K + j] (rows K..KD-1 are -inf), KD = wide_lane_stride(K).
 cudaError_t launch_wide_transpose(const float* logA, int K, float* AT, cudaStream_t st);
 void dense_stream_geometry(int K, int* KPM, int* cols);

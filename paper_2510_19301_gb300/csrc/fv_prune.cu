@@ -31,6 +31,8 @@
 #include <math_constants.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "fv_internal.cuh"
 #include "fv_launch.h"
 
@@ -47,15 +49,15 @@ __device__ __forceinline__ float ord_value(uint32_t k) {
   return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }
 
-// Padded row copy of logA (stride KP, columns beyond K -inf) and, per
-// column, the cutoff and the list of the rows above it, in ascending row
+// Padded row copy of logA (stride KP, columns beyond K -inf), its
+// column-major copy (rows K .. KD - 1 -inf) and, per column, the cutoff and the list of the rows above it, in ascending row
 // order: the largest cutoff with at most M rows above it, found by bisecting
 // the keys (a warp per column, VPL keys per lane in registers).
 // One CTA takes 8 adjacent columns, staged column-major in shared memory so
 // that global loads read whole 32-byte sectors.
 template <int VPL>
 __global__ void __launch_bounds__(256) prune_prep_kernel(const float* logA, int K, int KP, int M, float* Apad,
-                                                         float* lval, uint16_t* lrow, float* cut) {
+                                                         float* AT, float* lval, uint16_t* lrow, float* cut) {
   extern __shared__ float scol[];  // [8][32 * VPL + 4]
   constexpr int ST = 32 * VPL + 4;
   const int j0 = blockIdx.x * 8, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -67,6 +69,10 @@ __global__ void __launch_bounds__(256) prune_prep_kernel(const float* logA, int 
   }
   __syncthreads();
   const int j = j0 + warp;
+  if (j < K) {
+    const int KD = wide_lane_stride(K);
+    for (int i = lane; i < KD; i += 32) AT[(int64_t)j * KD + i] = i < K ? scol[warp * ST + i] : -CUDART_INF_F;
+  }
   uint32_t key[VPL];
 #pragma unroll
   for (int k = 0; k < VPL; ++k) {
@@ -925,8 +931,9 @@ struct TraceArgs {
   int64_t guess_cap;
   const WsHeader* hdr;
 };
-// TW warps of a CTA follow one chain, VPL rows of a column per thread.
-template <int VPL, int TW, bool BEAM>
+// TW warps of a CTA follow one chain, VPL rows of a column per thread; ROWS:
+// AT is logA itself (K <= 128: it stays in L1 whatever the order).
+template <int VPL, int TW, bool BEAM, bool ROWS>
 struct Tracer {
   static constexpr int AH = VPL <= 8 ? 4 : 2;  // delta rows loaded ahead
   static constexpr int NT = 32 * TW;
@@ -994,12 +1001,12 @@ struct Tracer {
   }
   // q_{t-1} from q_t; `x` holds delta_{t-1} and receives row t - 1 - AH
   __device__ __forceinline__ int step(int t, int q, Row& x) {
-    const float* col = AT + (int64_t)q * KD;
+    const float* col = AT + (ROWS ? q : q * (int64_t)KD);
     float v[VPL];
 #pragma unroll
     for (int k = 0; k < VPL; ++k) {
       const int i = BEAM ? x.i[k] : NT * k + tid;
-      v[k] = (BEAM ? i >= 0 : i < KD) ? __ldg(col + i) : -CUDART_INF_F;
+      v[k] = (BEAM ? i >= 0 : i < (ROWS ? K : KD)) ? __ldg(col + (ROWS ? i * K : i)) : -CUDART_INF_F;
     }
     float bv = -CUDART_INF_F;
     int bi = 0;
@@ -1050,7 +1057,7 @@ __device__ __forceinline__ int64_t guess_off(const TraceArgs& a, const Job& jb, 
   return jb.aux_off / ((int64_t)a.unit * a.seg) + b;
 }
 
-template <int VPL, int TW, bool BEAM>
+template <int VPL, int TW, bool BEAM, bool ROWS>
 __global__ void __launch_bounds__(32 * TW) prune_trace_kernel(TraceArgs a) {
   __shared__ uint2 part[2 * TW];
   if (a.hdr->status != 0) return;
@@ -1058,7 +1065,7 @@ __global__ void __launch_bounds__(32 * TW) prune_trace_kernel(TraceArgs a) {
   const Job jb = a.jobs[b];
   const int s = blockIdx.y, T = jb.T, K = a.K, lo = s * a.seg;
   if (lo >= T) return;
-  Tracer<VPL, TW, BEAM> tr;
+  Tracer<VPL, TW, BEAM, ROWS> tr;
   tr.init(a, jb, part);
   int32_t* path = a.paths + jb.path_off;
   const bool lead = threadIdx.x == 0;
@@ -1084,7 +1091,7 @@ __global__ void __launch_bounds__(32 * TW) prune_trace_kernel(TraceArgs a) {
   });
 }
 
-template <int VPL, int TW, bool BEAM>
+template <int VPL, int TW, bool BEAM, bool ROWS>
 __global__ void __launch_bounds__(32 * TW) prune_fix_kernel(TraceArgs a) {
   __shared__ uint2 part[2 * TW];
   if (a.hdr->status != 0) return;
@@ -1109,7 +1116,7 @@ __global__ void __launch_bounds__(32 * TW) prune_fix_kernel(TraceArgs a) {
       continue;
     }
     const int sb = s1 - (__ffs(m) - 1), lo = sb * a.seg, hi = lo + a.seg;
-    Tracer<VPL, TW, BEAM> tr;
+    Tracer<VPL, TW, BEAM, ROWS> tr;
     tr.init(a, jb, part);
     int q = __ldcg(path + hi);
     q = (unsigned)q < (unsigned)K ? q : 0;
@@ -1134,18 +1141,20 @@ int prune_pad(int K) { return K <= 256 ? 256 : K <= 512 ? 512 : K <= 1024 ? 1024
 int prune_list(int K) { return K <= 256 ? 6 : K <= 512 ? 12 : K <= 1024 ? 16 : 32; }
 // area: row copy, column-major copy, list values, cutoffs, list rows
 size_t prune_area_bytes(int K) {
+  if (K <= 128) return 0;  // (fv_small.cu needs none)
   const size_t KP = prune_pad(K), M = prune_list(K);
   return align_up((size_t)K * KP * 4) + align_up((size_t)K * wide_lane_stride(K) * 4) + align_up(KP * (M * 6 + 4));
 }
 
 template <int VPL>
-static cudaError_t launch_prep_cfg(const float* logA, int K, float* A, float* val, uint16_t* row, float* cut,
+static cudaError_t launch_prep_cfg(const float* logA, int K, float* A, float* at, float* val, uint16_t* row, float* cut,
                                    cudaStream_t st) {
   const size_t sm = 8 * (32 * VPL + 4) * sizeof(float);
   cudaError_t e =
       cudaFuncSetAttribute(prune_prep_kernel<VPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  prune_prep_kernel<VPL><<<prune_pad(K) / 8, 256, sm, st>>>(logA, K, prune_pad(K), prune_list(K), A, val, row, cut);
+  prune_prep_kernel<VPL><<<prune_pad(K) / 8, 256, sm, st>>>(logA, K, prune_pad(K), prune_list(K), A, at, val, row,
+                                                              cut);
   return cudaGetLastError();
 }
 
@@ -1163,24 +1172,26 @@ cudaError_t launch_prune_prep(const float* logA, int K, char* area, DenseArgs* a
   a->pr_row = row;
   a->pr_cut = cut;
   a->wide_AT = at;
-  cudaError_t e = launch_wide_transpose(logA, K, at, st);
-  if (e != cudaSuccess) return e;
-  if (K <= 256) return launch_prep_cfg<8>(logA, K, copy, val, row, cut, st);
-  if (K <= 512) return launch_prep_cfg<16>(logA, K, copy, val, row, cut, st);
-  if (K <= 1024) return launch_prep_cfg<32>(logA, K, copy, val, row, cut, st);
-  if (K <= 2048) return launch_prep_cfg<64>(logA, K, copy, val, row, cut, st);
-  return launch_prep_cfg<128>(logA, K, copy, val, row, cut, st);
+  if (K <= 256) return launch_prep_cfg<8>(logA, K, copy, at, val, row, cut, st);
+  if (K <= 512) return launch_prep_cfg<16>(logA, K, copy, at, val, row, cut, st);
+  if (K <= 1024) return launch_prep_cfg<32>(logA, K, copy, at, val, row, cut, st);
+  if (K <= 2048) return launch_prep_cfg<64>(logA, K, copy, at, val, row, cut, st);
+  return launch_prep_cfg<128>(logA, K, copy, at, val, row, cut, st);
 }
 
 // Clusters (CTAs for CL = 1) of a configuration resident at once; 0 where the
-// device does not take it.
+// device does not take it.  A property of the kernel and the device, asked
+// for once per device ordinal (a query and an attribute call cost several
+// microseconds of a short decode).
 template <int KP, int CL, int C, int G, bool RES, int M, bool BEAM>
 static int prune_resident(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
   using Cfg = PruneCfg<KP, CL, C, G, RES, M, BEAM>;
   static_assert(Cfg::smem + 1024 <= 227 * 1024, "one CTA per SM");
   static_assert(Cfg::W == 1 || G <= 15, "a named barrier per job group");
   auto kern = prune_fwd_kernel<KP, CL, C, G, RES, M, BEAM>;
-  int n = 0;
+  static std::atomic<int> known[64];  // per device, plus one
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
   const int nsm = device_sm_count();
   attr->id = cudaLaunchAttributeClusterDimension;
   attr->val.clusterDim.x = CL;
@@ -1191,6 +1202,7 @@ static int prune_resident(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
   cfg->dynamicSmemBytes = Cfg::smem;
   cfg->attrs = attr;
   cfg->numAttrs = 1;
+  if (known[dev].load() > 0) return known[dev].load() - 1;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem);
   if (e == cudaSuccess && CL > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess) {
@@ -1205,6 +1217,7 @@ static int prune_resident(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
     cudaGetLastError();
     return 0;
   }
+  known[dev].store(n + 1);
   return n;
 }
 
@@ -1267,32 +1280,34 @@ int prune_trace_seg(int64_t sum_T) {
   const int64_t s = (sum_T / 4096 + 15) / 16 * 16;
   return (int)(s < 48 ? 48 : s > 512 ? 512 : s);
 }
-// `unit`: table elements per step at least (128 for delta rows, the beam
-// table's row length)
+// `unit`: table elements per step at least (the smallest K for delta rows,
+// the beam table's row length)
 size_t prune_guess_bytes(uint64_t aux_elems, int32_t n_seq, int64_t sum_T, int32_t unit) {
   const uint64_t per = (uint64_t)unit * (uint64_t)prune_trace_seg(sum_T);
   return sizeof(int32_t) * (size_t)(aux_elems / per + (uint64_t)n_seq + 1ull);
 }
 
-template <int VPL, int TW, bool BEAM>
+template <int VPL, int TW, bool BEAM, bool ROWS>
 static cudaError_t launch_trace_cfg(const TraceArgs& t, int max_T, cudaStream_t st) {
   const dim3 grid(t.count, (max_T + t.seg - 1) / t.seg);
-  prune_trace_kernel<VPL, TW, BEAM><<<grid, 32 * TW, 0, st>>>(t);
-  if (grid.y > 1) prune_fix_kernel<VPL, TW, BEAM><<<t.count, 32 * TW, 0, st>>>(t);
+  prune_trace_kernel<VPL, TW, BEAM, ROWS><<<grid, 32 * TW, 0, st>>>(t);
+  if (grid.y > 1) prune_fix_kernel<VPL, TW, BEAM, ROWS><<<t.count, 32 * TW, 0, st>>>(t);
   return cudaGetLastError();
 }
 
 template <bool BEAM>
 static cudaError_t launch_trace(const TraceArgs& t, int n, int max_T, cudaStream_t st) {
-  if (n <= 256) return launch_trace_cfg<8, 1, BEAM>(t, max_T, st);
-  if (n <= 512) return launch_trace_cfg<16, 1, BEAM>(t, max_T, st);
-  if (n <= 1024) return launch_trace_cfg<16, 2, BEAM>(t, max_T, st);
-  if (n <= 2048) return launch_trace_cfg<16, 4, BEAM>(t, max_T, st);
-  return launch_trace_cfg<16, 8, BEAM>(t, max_T, st);
+  if (!BEAM && n <= 64) return launch_trace_cfg<2, 1, BEAM, true>(t, max_T, st);
+  if (!BEAM && n <= 128) return launch_trace_cfg<4, 1, BEAM, true>(t, max_T, st);
+  if (n <= 256) return launch_trace_cfg<8, 1, BEAM, false>(t, max_T, st);
+  if (n <= 512) return launch_trace_cfg<16, 1, BEAM, false>(t, max_T, st);
+  if (n <= 1024) return launch_trace_cfg<16, 2, BEAM, false>(t, max_T, st);
+  if (n <= 2048) return launch_trace_cfg<16, 4, BEAM, false>(t, max_T, st);
+  return launch_trace_cfg<16, 8, BEAM, false>(t, max_T, st);
 }
 
-cudaError_t launch_prune_trace(const DenseArgs& a, int32_t* guess, size_t guess_bytes, int64_t sum_T, int max_T,
-                               int32_t* paths, cudaStream_t st) {
+cudaError_t launch_prune_trace(const DenseArgs& a, int32_t* guess, size_t guess_bytes, int64_t sum_T, int unit,
+                               int max_T, int32_t* paths, cudaStream_t st) {
   if (a.order_count <= 0) return cudaSuccess;
   const bool beam = a.beam_B > 0;
   TraceArgs t;
@@ -1305,10 +1320,10 @@ cudaError_t launch_prune_trace(const DenseArgs& a, int32_t* guess, size_t guess_
   // (grid.y is at most 65535)
   if (max_T / t.seg > 32768) t.seg = (max_T / 32768 + 1) * t.seg;
   t.row = a.beam_stride;
-  t.unit = beam ? a.beam_stride : 128;
+  t.unit = unit;
   t.ids = a.beam_id;
   t.D = beam ? a.beam_val : a.pr_D;
-  t.AT = a.wide_AT;
+  t.AT = !beam && a.K <= 128 ? a.logA : a.wide_AT;
   t.qlast = a.qlast;
   t.paths = paths;
   t.guess = guess;

@@ -1,4 +1,6 @@
-// fv_small.cu -- the forward engine for small state spaces, K <= 128: a
+// fv_small.cu -- the forward engines for small state spaces, K <= 128.  Exact
+// decoding keeps values only where the workspace holds delta rows
+// (small_value_kernel, at the end).  Everything else: a
 // persistent grid of CTAs of KM threads (KM = 64 or 128, the class bound),
 // each running one job at a time from the launch's counter, for every
 // job kind of the slot engine: exact decoding with psi rows (Sec. III-A),
@@ -303,6 +305,166 @@ cudaError_t launch_small_forward(const DenseArgs& a, cudaStream_t st) {
   const int jobs = (a.kind == kJobVanilla || a.kind == kJobRoot) ? a.order_count : a.max_jobs;
   if (jobs <= 0) return cudaSuccess;
   return a.K <= 64 ? launch_small_class<64>(a, jobs, st) : launch_small_class<128>(a, jobs, st);
+}
+
+// ------------------------------------------------ exact decoding, values only
+// The same step keeping only the maximum: delta rows go to the workspace and
+// the backtrack recomputes the path's own argmaxima (fv_prune.cu), so two
+// candidates cost one packed add and one 3-input max instead of two adds,
+// compares and pairs of selects.  A thread per state holds its column as row
+// pairs.  Bound: the latency of a step (64 rows: an 8-deep chain of 3-input
+// maxima in each of four accumulators, one barrier).  Measured against the
+// argmax version above (GB300, whole calls): one K = 64 sequence of 1000
+// symbols 424 -> 317 us; 70 sequences of up to 19000 steps 9.4 -> 5.0 ms; us
+// per step of 1024 sequences, K = 64 1.31 -> 1.08, K = 128 3.68 -> 2.86.  Two
+// threads per state were slower (0.35 against 0.30 us per step at K = 64,
+// 0.64 against 0.50 at K = 128), four slower again.
+__device__ __forceinline__ void add2_max(float& m, unsigned long long d, unsigned long long w) {
+  asm("{\n\t.reg .b64 c;\n\t.reg .f32 lo, hi;\n\tadd.rn.f32x2 c, %1, %2;\n\tmov.b64 {lo, hi}, c;\n\t"
+      "max.f32 %0, %0, lo, hi;\n\t}"
+      : "+f"(m)
+      : "l"(d), "l"(w));
+}
+
+template <int KM>
+__global__ void __launch_bounds__(KM + 32) small_value_kernel(DenseArgs a) {
+  constexpr int BA = 8, AH = 2 * BA;  // emission rows: a batch on its way, a ring of two
+  __shared__ __align__(16) float sd[2][KM];
+  __shared__ __align__(16) float sE[AH][KM];  // E_t in slot t % AH
+  if (a.hdr->status != 0) return;  // an earlier kernel recorded an error
+  const int K = a.K, tid = threadIdx.x, j = tid;
+  const bool own = j < K;
+  const int b = a.order[a.order_begin + (int)blockIdx.x];
+  const Job jb = a.jobs[b];
+  const int T = jb.T;
+  if (T < 1) return;
+  // The last warp fetches the emission rows, a batch of BA steps ahead in its
+  // registers and the next in the ring: a step never waits for memory.  (Rows
+  // prefetched in the workers' own registers were waited for one step later,
+  // as the loads share a scoreboard: 0.47 us per step where E came from
+  // memory, against 0.27 from L2; a ring of cp.async cost 0.15 us per step.)
+  if (tid >= KM) {
+    const int lane = tid & 31;
+    const bool dense = a.emit == FV_EMIT_DENSE;
+    float v[BA][KM / 32];
+    int xs = 0;  // discrete: lane l holds the symbol of row l of the batch after v
+    auto symbols = [&](int t) {
+      if (!dense && lane < BA && t + lane < T) xs = __ldg(a.obs + jb.e_off + t + lane);
+    };
+    auto load = [&](int t) {
+#pragma unroll
+      for (int r = 0; r < BA; ++r) {
+        const int x = dense ? 0 : __shfl_sync(0xffffffffu, xs, r);
+#pragma unroll
+        for (int c = 0; c < KM / 32; ++c) {
+          const int jj = 32 * c + lane;
+          if (t + r < T && jj < K)
+            v[r][c] = dense ? __ldg(a.E + jb.e_off + (int64_t)(t + r) * K + jj) : __ldg(a.logB + (int64_t)jj * a.V + x);
+        }
+      }
+    };
+    auto store = [&](int t) {
+#pragma unroll
+      for (int r = 0; r < BA; ++r)
+#pragma unroll
+        for (int c = 0; c < KM / 32; ++c) sE[(t + r) % AH][32 * c + lane] = v[r][c];
+    };
+#pragma unroll
+    for (int r = 0; r < BA; ++r)
+#pragma unroll
+      for (int c = 0; c < KM / 32; ++c) v[r][c] = 0.f;
+    symbols(0);
+    load(0);
+    symbols(BA);
+    store(0);
+    load(BA);
+    symbols(2 * BA);
+    __syncthreads();
+    for (int t = 0; t < T; ++t) {
+      if (t % BA == 0) {
+        store(t + BA);  // (their slots were read before step t)
+        load(t + 2 * BA);
+        symbols(t + 3 * BA);
+      }
+      __syncthreads();
+    }
+    return;
+  }
+  // row pairs of the column; rows and states beyond K are -inf
+  unsigned long long A[KM / 2];
+#pragma unroll
+  for (int i = 0; i < KM / 2; ++i) {
+    const int r = 2 * i;
+    const float lo = (own && r < K) ? __ldg(a.logA + (int64_t)r * K + j) : -CUDART_INF_F;
+    const float hi = (own && r + 1 < K) ? __ldg(a.logA + (int64_t)(r + 1) * K + j) : -CUDART_INF_F;
+    A[i] = ((unsigned long long)__float_as_uint(hi) << 32) | (unsigned long long)__float_as_uint(lo);
+  }
+  __syncthreads();
+  float* dt = a.pr_D + jb.aux_off + j;
+  int cur = 0;
+#pragma unroll 2
+  for (int t = 0; t < T; ++t) {
+    const float e = sE[t % AH][j];
+    float dval;
+    if (t == 0) {
+      dval = own ? __fadd_rn(__ldg(a.log_pi + j), e) : -CUDART_INF_F;
+    } else {
+      const ulonglong2* dv = reinterpret_cast<const ulonglong2*>(sd[cur]);
+      float m[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
+#pragma unroll
+      for (int i = 0; i < KM / 4; ++i) {
+        const ulonglong2 x = dv[i];
+        add2_max(m[(2 * i) & 3], x.x, A[2 * i]);
+        add2_max(m[(2 * i + 1) & 3], x.y, A[2 * i + 1]);
+      }
+      const float bv = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+      dval = __fadd_rn(bv, e);  // (-inf beyond K)
+      if (dval == 0.f && bv == 0.f && __float_as_uint(e) == 0x80000000u && own) {
+        // a zero plus E = -0 has the sign of the kept candidate's zero, the
+        // lowest maximising row's
+        for (int i = 0; i < K; ++i) {
+          const float c = __fadd_rn(sd[cur][i], __ldg(a.logA + (int64_t)i * K + j));
+          if (c == 0.f) {
+            dval = __fadd_rn(c, e);
+            break;
+          }
+        }
+      }
+    }
+    sd[cur ^ 1][j] = dval;
+    if (own) __stcs(dt, dval);
+    dt += K;
+    __syncthreads();
+    cur ^= 1;
+  }
+  if (tid < 32) {
+    // termination: q_{T-1} = lowest argmax_j delta_{T-1}[j], score = delta_{T-1}[q]
+    float v = sd[cur][tid];
+    int qi = tid;
+#pragma unroll
+    for (int k = 1; k < KM / 32; ++k) {
+      const float vk = sd[cur][tid + 32 * k];
+      if (vk > v) { v = vk; qi = tid + 32 * k; }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float ov = __shfl_xor_sync(0xffffffffu, v, o);
+      const int oq = __shfl_xor_sync(0xffffffffu, qi, o);
+      if (ov > v || (ov == v && oq < qi)) { v = ov; qi = oq; }
+    }
+    if (tid == 0) {
+      a.qlast[b] = qi;
+      a.scores[b] = sd[cur][qi];
+    }
+  }
+}
+
+cudaError_t launch_small_values(const DenseArgs& a, cudaStream_t st) {
+  if (a.K > 128) return cudaErrorInvalidValue;
+  if (a.order_count <= 0) return cudaSuccess;
+  if (a.K <= 64) small_value_kernel<64><<<a.order_count, 64 + 32, 0, st>>>(a);
+  else small_value_kernel<128><<<a.order_count, 128 + 32, 0, st>>>(a);
+  return cudaGetLastError();
 }
 
 }  // namespace fv
