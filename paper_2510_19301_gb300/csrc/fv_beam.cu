@@ -923,6 +923,31 @@ __global__ void __launch_bounds__(kCBThreads, 1) beam_csr_cluster_kernel(BeamArg
     if (tid < kCB) dsmem_st_u32(dsmem_addr(&cnt[which * kCB + (int)rank], (uint32_t)tid), (uint32_t)v);
   };
 
+  // ---- the select by score bins around the threshold expected from the last
+  // steps (every CTA holds the same expectation): one histogram over the
+  // cluster finds the bin of the W-th candidate, the few candidates of that
+  // bin go to every CTA and are ranked there.  Two cluster barriers where the
+  // radix passes below take six; those remain for the first step and for a
+  // step whose threshold lies outside the bins or shares its bin with more
+  // than kTies candidates.
+  constexpr int kTies = 128;
+  __shared__ float2 tie[kCB][kTies];
+  __shared__ int s_tn, s_take[kCB];
+  __shared__ float s_tv;
+  __shared__ int s_ti;
+  bool have = false;
+  float pred = 0.f, grow = 0.f, last = 0.f, scale = 16.f;
+  auto bin_of = [&](float c) -> int {
+    const float x = __fadd_rn(__fadd_rn(pred, -c) * scale, 128.f);
+    return x > 0.f ? (x < 255.f ? (int)x : 255) : 0;
+  };
+  auto expect = [&](float thr_v) {
+    if (have) grow = 0.75f * grow + 0.25f * __fadd_rn(thr_v, -last);
+    last = thr_v;
+    pred = __fadd_rn(thr_v, grow);
+    have = fabsf(pred) < 1e30f;
+  };
+
   // top-W of the list (n entries; values lval, ids lid, ascending) over the
   // whole cluster -> beam buffer q at its global positions; returns the new
   // beam size (identical in every CTA).  Writes backpointers of step t when
@@ -930,6 +955,143 @@ __global__ void __launch_bounds__(kCBThreads, 1) beam_csr_cluster_kernel(BeamArg
   auto select_gather = [&](int n, int W, int q, int bp_t, bool from_keys, const Job& jb) -> int {
     const int e0 = min(n, tid * ((n + (int)blockDim.x - 1) / (int)blockDim.x));
     const int e1 = min(n, e0 + (n + (int)blockDim.x - 1) / (int)blockDim.x);
+    if (have) {
+      int* h = hist;
+      for (int k = tid; k < 256; k += blockDim.x) {
+        h[k] = 0;
+        htot[k] = 0;
+      }
+      if (tid == 0) s_tn = 0;
+      if (tid < kCB) s_take[tid] = 0;
+      __syncthreads();
+      for (int e = tid; e < n; e += blockDim.x) {
+        const float c = lval[e];
+        if (isfinite(c)) atomicAdd(&h[bin_of(c)], 1);
+      }
+      cluster_sync_all();  // every rank's histogram is complete
+      for (int x = tid; x < 256 * kCB; x += blockDim.x) {
+        const int d = x & 255, r = x >> 8;
+        const int v = (int)dsmem_ld_u32(dsmem_addr(&h[d], (uint32_t)r));
+        if (v) atomicAdd(&htot[d], v);
+      }
+      __syncthreads();
+      if (tid < 32) {
+        int hv[8], sum = 0, own = 0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          hv[u] = htot[8 * lane + u];
+          sum += hv[u];
+        }
+        int incl = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += y;
+        }
+        const int total = __shfl_sync(0xffffffffu, incl, 31);
+        int bb = 256, left = 0, inb = 0, acc = incl - sum;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          if (total > W && acc < W && W <= acc + hv[u]) {
+            bb = 8 * lane + u;
+            left = W - acc;
+            inb = hv[u];
+          }
+          acc += hv[u];
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, bb < 256);
+        if (m) {
+          const int src = __ffs(m) - 1;
+          bb = __shfl_sync(0xffffffffu, bb, src);
+          left = __shfl_sync(0xffffffffu, left, src);
+          inb = __shfl_sync(0xffffffffu, inb, src);
+          // this rank's candidates in the bins above
+#pragma unroll
+          for (int u = 0; u < 8; ++u) own += 8 * lane + u < bb ? h[8 * lane + u] : 0;
+          for (int o = 16; o > 0; o >>= 1) own += __shfl_xor_sync(0xffffffffu, own, o);
+        }
+        if (lane == 0) {
+          misc[0] = bb;
+          misc[1] = left;
+          misc[2] = inb;
+          misc[3] = own;
+          misc[4] = total;
+        }
+      }
+      __syncthreads();
+      const int bb = misc[0], left = misc[1], inb = misc[2], own_gt = misc[3], total = misc[4];
+      if (total == 0) return 0;
+      if (bb > 0 && bb < 255 && inb <= kTies) {
+        for (int e = tid; e < n; e += blockDim.x) {
+          const float c = lval[e];
+          if (isfinite(c) && bin_of(c) == bb) {
+            const int x = atomicAdd(&s_tn, 1);
+            for (int q2 = 0; q2 < kCB; ++q2) {
+              const uint32_t to = dsmem_addr(&tie[rank][x], (uint32_t)q2);
+              dsmem_st_f32(to, c);
+              dsmem_st_u32(to + 4u, (uint32_t)lid[e]);
+            }
+          }
+        }
+        __syncthreads();
+        publish(1, own_gt);
+        publish(2, s_tn);
+        cluster_sync_all();  // every rank's counts and candidates of the bin are here
+        if (tid < inb) {
+          // candidate tid of the bin, ranks in order
+          int r = 0, x = tid;
+          while (x >= cnt[2 * kCB + r]) x -= cnt[2 * kCB + r++];
+          const float2 me = tie[r][x];
+          const int id = __float_as_int(me.y);
+          int ahead = 0;
+          for (int r2 = 0; r2 < kCB; ++r2)
+            for (int y = 0; y < cnt[2 * kCB + r2]; ++y) {
+              const float2 o = tie[r2][y];
+              ahead += o.x > me.x || (o.x == me.x && __float_as_int(o.y) < id);
+            }
+          if (ahead < left) atomicAdd(&s_take[r], 1);
+          if (ahead == left - 1) {
+            s_tv = me.x;
+            s_ti = id;
+          }
+        }
+        __syncthreads();
+        const float tv = s_tv;
+        const int ti = s_ti;
+        int win_before = 0;
+        for (int r = 0; r < (int)rank; ++r) win_before += cnt[1 * kCB + r] + s_take[r];
+        auto wins = [&](int e) -> bool {
+          const float c = lval[e];
+          if (!isfinite(c)) return false;
+          const int d = bin_of(c);
+          return d < bb || (d == bb && (c > tv || (c == tv && lid[e] <= ti)));
+        };
+        int mine = 0;
+        for (int e = e0; e < e1; ++e) mine += wins(e) ? 1 : 0;
+        int tot;
+        int o = win_before + block_scan(mine, red, &tot);
+        for (int e = e0; e < e1; ++e) {
+          if (!wins(e)) continue;
+          const int j = lid[e];
+          bid[q][o] = j;
+          bval[q][o] = lval[e];
+          if (bp_t >= 0) {
+            const int sl = from_keys ? (int)(0xFFFFFFFFull - (keys[j] & 0xFFFFFFFFull)) : 0;
+            a.bp_id[jb.aux_off + (int64_t)bp_t * a.Wcap + o] = j;
+            a.bp_src[jb.aux_off + (int64_t)bp_t * a.Wcap + o] = sl;
+          }
+          ++o;
+        }
+        // bins as fine as a handful of candidates in one
+        if (inb > 16) scale = fminf(1.25f * scale, 1e20f);
+        else if (inb < 3) scale = fmaxf(0.9f * scale, 1e-20f);
+        expect(tv);
+        __syncthreads();  // every thread has read its winners' keys before any is cleared
+        return W;
+      }
+      if (bb == 0 || bb == 255) scale = fmaxf(0.5f * scale, 1e-20f);
+      else if (inb > kTies) scale = fminf(2.f * scale, 1e20f);
+      __syncthreads();
+    }
     int fin = 0;
     for (int e = e0; e < e1; ++e) fin += isfinite(lval[e]) ? 1 : 0;
     fin = block_sum(fin, red);
@@ -996,6 +1158,7 @@ __global__ void __launch_bounds__(kCBThreads, 1) beam_csr_cluster_kernel(BeamArg
       }
       thr = prefix;
       need_eq = remaining;
+      expect(ord_value(thr));
     }
     // winners of this rank: keys above the threshold, and keys equal to it
     // while the lower ranks have not taken the needed number
@@ -1068,6 +1231,8 @@ __global__ void __launch_bounds__(kCBThreads, 1) beam_csr_cluster_kernel(BeamArg
       __syncthreads();
     }
     int p = 0;
+    have = false;  // (the first step's threshold has no predecessor)
+    grow = 0.f;
     int nb = select_gather(n, W, p, 0, false, jb);
     cluster_sync_all();  // beam 0 is complete in global memory
     bool infeasible = nb == 0;
