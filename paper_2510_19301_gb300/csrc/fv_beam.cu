@@ -834,20 +834,27 @@ __global__ void __launch_bounds__(kBeamThreads, 1) beam_kernel(BeamArgs a) {
 // kCB CTAs (kJobBeam, large K).  The single-CTA kernel above keeps one SM
 // busy per sequence and is bound by the latency of each step's phases; here
 // every phase is split kCB ways:
-//  * scatter: CTA r relaxes the out-edges of its share of the beam entries
-//    (64-bit atomicMax on the cluster's key array in global memory, the
-//    same keys as above) and marks each target in the bitmap of the CTA
-//    that owns the target's id range (distributed shared memory);
+//  * scatter: CTA r relaxes the out-edges of the beam entries of its own id
+//    range, still in its shared memory (64-bit atomicMax on the cluster's
+//    key array in global memory, the same keys as above), and marks each
+//    target in the bitmap of the CTA that owns the target's id range
+//    (distributed shared memory);
 //  * candidates: CTA r lists the touched targets of its id range (ids
-//    [r R, (r+1) R)) in shared memory, in id order, with c_j = M_j + E_t[j];
-//  * top-B select: the MSB radix select of the single-CTA kernel with every
-//    pass's 256-bin histogram summed over the cluster (each CTA reads the
-//    others' histograms through distributed shared memory), so every CTA
-//    takes the same threshold; keys equal to the threshold go to the lowest
-//    ids first, i.e. to the lower ranks first;
+//    [r R, (r+1) R)) in shared memory, in id order, then forms c_j = M_j +
+//    E_t[j] and the source slots with the list strided over the block, and
+//    clears the keys it has read;
+//  * top-B select: bins of the score around the expected threshold, summed
+//    over the cluster, then the candidates of the B-th one's bin ranked in
+//    every CTA (below); the MSB radix select of the single-CTA kernel with
+//    every pass's histogram summed over the cluster is the fallback;
 //  * gather: each CTA learns how many winners the lower ranks hold and
 //    writes its own at that offset, in id order -- the next beam, sorted by
 //    id, in global memory, with the step's backpointers.
+// Three cluster barriers per step (scatter, bins, ranked bin).  Bound: their
+// latency and that of the graph's loads.  Measured (GB300, K = 65536, 32
+// successors, 8 sequences, us per step at B = 128 / 512 / 2048): 22.4 / 27.0 /
+// 43.7 with radix passes (eight barriers), 18.3 / 22.6 / 38.9 with bins, 11.5 /
+// 17.2 / 34.5 with the scatter from shared memory and the strided list.
 // Result: the same beams, paths and scores as the single-CTA kernel.
 constexpr int kCB = 8;              // CTAs per sequence (portable cluster size)
 constexpr int kCBThreads = 1024;
@@ -863,9 +870,9 @@ __device__ inline uint32_t dsmem_ld_u32(uint32_t addr) {
 
 // ids per rank, its bitmap words and the shared-memory layout
 __host__ __device__ inline int cb_range(int K) { return (K + kCB - 1) / kCB; }
-__host__ __device__ inline size_t cb_smem_bytes(int K) {
-  const size_t R = (size_t)cb_range(K), bm = ((R + 31) / 32 + 3) / 4 * 4;
-  return 4 * (bm + 2 * R + 3 * 256 + 4 * kCB + 16);
+__host__ __device__ inline size_t cb_smem_bytes(int K, int W) {
+  const size_t R = (size_t)cb_range(K), bm = ((R + 31) / 32 + 3) / 4 * 4, w = (size_t)W < R ? (size_t)W : R;
+  return 4 * (bm + 3 * R + 2 * w + 3 * 256 + 4 * kCB + 16);
 }
 
 __global__ void __launch_bounds__(kCBThreads, 1) beam_csr_cluster_kernel(BeamArgs a) {
@@ -880,7 +887,11 @@ __global__ void __launch_bounds__(kCBThreads, 1) beam_csr_cluster_kernel(BeamArg
   uint32_t* bitmap = csm;                                            // [bm_words] touched, local ids
   float* lval = reinterpret_cast<float*>(bitmap + bm_words);         // [R] listed candidate values
   int32_t* lid = reinterpret_cast<int32_t*>(lval + R);               // [R] their ids, ascending
-  int* hist = reinterpret_cast<int*>(lid + R);                       // [2][256] this CTA's histograms
+  int32_t* lsrc = lid + R;                                           // [R] their source slots
+  const int Wl = min(min(a.Wcap, a.Bcap), R);
+  int32_t* wid = lsrc + R;                                           // [Wl] this rank's beam entries
+  float* wval = reinterpret_cast<float*>(wid + Wl);
+  int* hist = reinterpret_cast<int*>(wval + Wl);                     // [2][256] this CTA's histograms
   int* cnt = hist + 512;                                             // [4][kCB] counts from every rank
   int* htot = cnt + 4 * kCB;                                         // [256] the cluster's histogram
   const int cl = blockIdx.x / kCB, ncl = gridDim.x / kCB;
@@ -947,6 +958,9 @@ __global__ void __launch_bounds__(kCBThreads, 1) beam_csr_cluster_kernel(BeamArg
     pred = __fadd_rn(thr_v, grow);
     have = fabsf(pred) < 1e30f;
   };
+
+  // this rank's entries of the beam: slots loc_base .. loc_base + loc_n
+  int loc_base = 0, loc_n = 0;
 
   // top-W of the list (n entries; values lval, ids lid, ascending) over the
   // whole cluster -> beam buffer q at its global positions; returns the new
@@ -1069,13 +1083,17 @@ __global__ void __launch_bounds__(kCBThreads, 1) beam_csr_cluster_kernel(BeamArg
         for (int e = e0; e < e1; ++e) mine += wins(e) ? 1 : 0;
         int tot;
         int o = win_before + block_scan(mine, red, &tot);
+        loc_base = win_before;
+        loc_n = tot;
         for (int e = e0; e < e1; ++e) {
           if (!wins(e)) continue;
           const int j = lid[e];
+          wid[o - win_before] = j;
+          wval[o - win_before] = lval[e];
           bid[q][o] = j;
           bval[q][o] = lval[e];
           if (bp_t >= 0) {
-            const int sl = from_keys ? (int)(0xFFFFFFFFull - (keys[j] & 0xFFFFFFFFull)) : 0;
+            const int sl = from_keys ? lsrc[e] : 0;
             a.bp_id[jb.aux_off + (int64_t)bp_t * a.Wcap + o] = j;
             a.bp_src[jb.aux_off + (int64_t)bp_t * a.Wcap + o] = sl;
           }
@@ -1085,7 +1103,7 @@ __global__ void __launch_bounds__(kCBThreads, 1) beam_csr_cluster_kernel(BeamArg
         if (inb > 16) scale = fminf(1.25f * scale, 1e20f);
         else if (inb < 3) scale = fmaxf(0.9f * scale, 1e-20f);
         expect(tv);
-        __syncthreads();  // every thread has read its winners' keys before any is cleared
+        __syncthreads();  // this rank's entries are complete
         return W;
       }
       if (bb == 0 || bb == 255) scale = fmaxf(0.5f * scale, 1e-20f);
@@ -1190,6 +1208,8 @@ __global__ void __launch_bounds__(kCBThreads, 1) beam_csr_cluster_kernel(BeamArg
     const int take_eq = min(max(take_rank - eq_before_loc, 0), n_eq);
     int tot;
     int o = win_before + block_scan(n_gt + take_eq, red, &tot);
+    loc_base = win_before;
+    loc_n = tot;
     int eq_seen = 0;
     for (int e = e0; e < e1; ++e) {
       const float c = lval[e];
@@ -1199,16 +1219,18 @@ __global__ void __launch_bounds__(kCBThreads, 1) beam_csr_cluster_kernel(BeamArg
       if (!take && u == thr) take = (eq_seen++ < take_eq);
       if (!take) continue;
       const int j = lid[e];
+      wid[o - win_before] = j;
+      wval[o - win_before] = c;
       bid[q][o] = j;
       bval[q][o] = c;
       if (bp_t >= 0) {
-        const int sl = from_keys ? (int)(0xFFFFFFFFull - (keys[j] & 0xFFFFFFFFull)) : 0;
+        const int sl = from_keys ? lsrc[e] : 0;
         a.bp_id[jb.aux_off + (int64_t)bp_t * a.Wcap + o] = j;
         a.bp_src[jb.aux_off + (int64_t)bp_t * a.Wcap + o] = sl;
       }
       ++o;
     }
-    __syncthreads();  // every thread has read its winners' keys before any is cleared
+    __syncthreads();  // this rank's entries are complete
     return nb;
   };
 
@@ -1234,7 +1256,6 @@ __global__ void __launch_bounds__(kCBThreads, 1) beam_csr_cluster_kernel(BeamArg
     have = false;  // (the first step's threshold has no predecessor)
     grow = 0.f;
     int nb = select_gather(n, W, p, 0, false, jb);
-    cluster_sync_all();  // beam 0 is complete in global memory
     bool infeasible = nb == 0;
     for (int t = 1; t < T && !infeasible; ++t) {
       // the next step's emission row goes to L2 while this one is used
@@ -1242,50 +1263,54 @@ __global__ void __launch_bounds__(kCBThreads, 1) beam_csr_cluster_kernel(BeamArg
         const float* row = a.E + jb.e_off + (int64_t)(t + 1) * K;
         if (((uintptr_t)row & 15u) == 0) prefetch_l2_bulk(row, (uint32_t)K * 4u);
       }
-      // ---- scatter this rank's share of the beam entries
-      const int s0 = (int)(((int64_t)nb * rank) / kCB), s1 = (int)(((int64_t)nb * (rank + 1)) / kCB);
-      for (int k = s0 + warp; k < s1; k += nwarp) {
-        const int i = bid[p][k];
-        const float v = bval[p][k];
+      // ---- relax the out-edges of this rank's own entries (still in its
+      // shared memory; every rank's keys and bitmap of the last step were
+      // cleared before the barriers of its select)
+      for (int k = warp; k < loc_n; k += nwarp) {
+        const int i = wid[k];
+        const float v = wval[k];
+        const unsigned slot = (unsigned)(loc_base + k);
         for (int e = a.row_ptr[i] + lane; e < a.row_ptr[i + 1]; e += 32) {
           const int j = a.col[e];
           const float c = __fadd_rn(v, a.val[e]);
-          const unsigned long long key = ((unsigned long long)ord_key(c) << 32) | (0xFFFFFFFFull - (unsigned)k);
+          const unsigned long long key = ((unsigned long long)ord_key(c) << 32) | (0xFFFFFFFFull - slot);
           atomicMax(&keys[j], key);
           const int ow = j / R, jl = j - ow * R;
           dsmem_red_or(dsmem_addr(&bitmap[jl >> 5], (uint32_t)ow), 1u << (jl & 31));
         }
       }
-      cluster_sync_all();  // keys and bitmaps of this step are complete
-      // ---- candidates of this rank's ids, listed in id order
+      cluster_sync_all();  // keys and bitmaps of this step, and the beam before it, are complete
+      // ---- candidates of this rank's ids, listed in id order; then their
+      // keys and emission scores, the same number of loads for every thread
       {
         int c_n = 0;
         for (int x = t0; x < t1; ++x) c_n += (bitmap[x >> 5] >> (x & 31)) & 1u;
         int tot;
         int o = block_scan(c_n, red, &tot);
-        for (int x = t0; x < t1; ++x) {
-          if (!((bitmap[x >> 5] >> (x & 31)) & 1u)) continue;
-          const int j = j_lo + x;
+        for (int x = t0; x < t1; ++x)
+          if ((bitmap[x >> 5] >> (x & 31)) & 1u) lid[o++] = j_lo + x;
+        n = tot;
+        __syncthreads();
+        for (int w = tid; w < bm_words; w += blockDim.x) bitmap[w] = 0u;
+        for (int e = tid; e < n; e += blockDim.x) {
+          const int j = lid[e];
+          const float em = beam_emit(a, jb, t, j);
           const unsigned long long key = keys[j];
           const int sl = (int)(0xFFFFFFFFull - (key & 0xFFFFFFFFull));
           float m = ord_value((uint32_t)(key >> 32));
           if (m == 0.0f) m = __fadd_rn(bval[p][sl], beam_csr_w(a, bid[p][sl], j));
-          lval[o] = __fadd_rn(m, beam_emit(a, jb, t, j));
-          lid[o] = j;
-          ++o;
+          lval[e] = __fadd_rn(m, em);
+          lsrc[e] = sl;
+          keys[j] = 0ull;
         }
-        n = tot;
         __syncthreads();
       }
       const int np = p ^ 1;
       nb = select_gather(n, W, np, t, true, jb);
-      // ---- clear this rank's keys and bitmap
-      for (int e = tid; e < n; e += blockDim.x) keys[lid[e]] = 0ull;
-      for (int w = tid; w < bm_words; w += blockDim.x) bitmap[w] = 0u;
-      cluster_sync_all();  // the next beam is complete; keys and bitmaps are clear
       p = np;
       if (nb == 0) infeasible = true;
     }
+    cluster_sync_all();  // the last beam is complete in global memory
     if (!infeasible) {
       if (rank == 0 && tid == 0) {
         int kb = 0;  // best final entry: highest score, lowest id
@@ -1877,7 +1902,7 @@ static int launch_beam_cluster(const BeamArgs& a, int max_jobs, cudaStream_t st,
   *err = cudaSuccess;
   if (a.trans != FV_TRANS_CSR || a.kind != kJobBeam || a.static_beam || a.K < 8192) return 1;
   if (a.Wcap < 64) return 1;  // narrow beams: one CTA per sequence has less per-step latency
-  const size_t smem = cb_smem_bytes(a.K);
+  const size_t smem = cb_smem_bytes(a.K, a.Wcap < a.Bcap ? a.Wcap : a.Bcap);
   if (smem > (size_t)200 * 1024) return 1;
   int clusters = a.max_ctas / kCB;
   if (max_jobs < clusters) clusters = max_jobs;
