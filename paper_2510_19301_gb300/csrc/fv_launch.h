@@ -113,6 +113,9 @@ struct DenseArgs {
   // restarts segment tasks from those checkpoints and writes the segment's
   // backpointer rows after them (`psi` = the same area as uint16)
   int32_t ckpt;
+  // K <= 128, kJobLeaf: tasks of at most `direct` rows (n - m) keep their
+  // backpointer rows in shared memory and write their path (0: rows to psi)
+  int32_t direct;
   const float2* Ap;           // streamed configurations: row-pair copy of logA
   int64_t ap_stride;          // float2 per row pair of Ap
   float* snap_scratch;        // streamed configurations: sub snapshots [clusters][S][rows]
@@ -249,6 +252,9 @@ cudaError_t launch_prune_trace(const DenseArgs& a, int32_t* guess, size_t guess_
                                int max_T, int32_t* paths, cudaStream_t st);
 bool prune_beam_wins(int K, int64_t sum_T, int max_T, bool alone);
 cudaError_t launch_prune_beam(const DenseArgs& a, bool alone, cudaStream_t st);
+// FLASH tasks of at most this many backpointer rows are solved in one launch
+// (K <= 128 on the default engine; 0: not there)
+int dense_direct_rows(int K, bool no_tune);
 bool dense_prune_K(int K);
 bool dense_uses_prune(int K, bool no_tune, bool withhold);
 // exact decoding at K <= 128, values only: delta rows to a.pr_D (fv_small.cu)

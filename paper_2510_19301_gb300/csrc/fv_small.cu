@@ -64,6 +64,8 @@ __global__ void __launch_bounds__(KM * TPC, VAN ? (KM <= 64 ? 6 : 2) : (KM <= 64
   __shared__ uint16_t smid[2][KM];  // MidState_{t-1}, MidState_t
   __shared__ float ssnap[KM];       // sub jobs: delta_{tmid}
   extern __shared__ float sB_dyn[];
+  // direct tasks: the segment's backpointer rows, [row][KM], after the table
+  uint8_t* spsi = reinterpret_cast<uint8_t*>(sB_dyn + (small_stage_logB<KM>(a) ? (size_t)a.V * KM : 0));
   if (a.hdr->status != 0) return;  // an earlier kernel recorded an error
   const int kind = VAN ? (int)kJobVanilla : a.kind, K = a.K, tid = threadIdx.x;
   const int j = tid / TPC, h = tid % TPC, r0 = h * RH;  // state, row share, its first row
@@ -107,6 +109,11 @@ __global__ void __launch_bounds__(KM * TPC, VAN ? (KM <= 64 ? 6 : 2) : (KM <= 64
     const Job jb = a.jobs[b];
     const int T = jb.T;
     if (T < 1 || n < m) return;
+    if (!VAN && a.direct && n - m > a.direct) {
+      // the lengths on the device are not the host's: no room for the rows
+      if (tid == 0) set_status(a.hdr, FV_EINVAL, (uint32_t)b);
+      return;
+    }
     if constexpr (VAN) load_column();  // (one job per CTA)
     if (kind == kJobRoot || (kind == kJobLeaf && a.ckpt)) Pe = a.ckpt ? ckpt_count(T, a.P) : flash_pe(T, a.P);
     if (from_tasks && !a.ckpt) {
@@ -190,7 +197,9 @@ __global__ void __launch_bounds__(KM * TPC, VAN ? (KM <= 64 ? 6 : 2) : (KM <= 64
           if (other) { bv = ov; g = og; }
         }
         dval = own ? __fadd_rn(bv, e) : -CUDART_INF_F;
-        if (lead && own && (kind == kJobVanilla || kind == kJobLeaf)) {
+        if (!VAN && a.direct) {
+          if (lead) spsi[(t - m - 1) * KM + j] = (uint8_t)g;
+        } else if (lead && own && (kind == kJobVanilla || kind == kJobLeaf)) {
           const int64_t row = kind == kJobVanilla ? jb.aux_off + (int64_t)t * K
                               : a.ckpt        ? 2 * (jb.aux_off + (int64_t)Pe * K) + (int64_t)(t - m - 1) * K
                                               : (int64_t)(pad + t - m - 1) * K;
@@ -243,6 +252,16 @@ __global__ void __launch_bounds__(KM * TPC, VAN ? (KM <= 64 ? 6 : 2) : (KM <= 64
         a.qlast[b] = qi;
         a.scores[b] = sd[cur][qi];
       }
+    } else if (!VAN && a.direct && tid == 0) {
+      // q_{t-1} = psi_t[q_t] from the known q_n (the last step's barrier
+      // completed the rows; the next job starts behind a barrier)
+      int32_t* path = a.paths + jb.path_off;
+      int q = q_n;
+      for (int t = n; t > m; --t) {
+        q = spsi[(t - m - 1) * KM + q];
+        q = q < K ? q : 0;
+        path[t - 1] = q;
+      }
     } else if (kind == kJobSub && tid == 0) {
       // Alg. 2 output: q*_{tmid} = MidState_n[q*_n]; its delta from the snapshot
       int q = smid[cur][q_n];
@@ -266,6 +285,12 @@ __global__ void __launch_bounds__(KM * TPC, VAN ? (KM <= 64 ? 6 : 2) : (KM <= 64
   }
 }
 
+// dynamic shared memory: the staged symbol table, and the rows of direct tasks
+template <int KM>
+static size_t small_smem(const DenseArgs& a) {
+  return (small_stage_logB<KM>(a) ? (size_t)a.V * KM * sizeof(float) : 0) + (size_t)a.direct * KM;
+}
+
 // exact decoding: one CTA per sequence; other kinds: a persistent grid of
 // the CTAs resident at once (per instance), at most one per job
 // CTAs of the instance resident at once on the device (0 on an error)
@@ -283,7 +308,7 @@ static int small_resident(size_t sm) {
 
 template <int KM, bool VAN, int TPC>
 static cudaError_t launch_small_cfg(const DenseArgs& a, int jobs, int resident, cudaStream_t st) {
-  const size_t sm = small_stage_logB<KM>(a) ? (size_t)a.V * KM * sizeof(float) : 0;
+  const size_t sm = small_smem<KM>(a);
   if (resident < 1) return cudaErrorInvalidConfiguration;
   const int grid = VAN ? jobs : (jobs < resident ? jobs : resident);
   small_fwd_kernel<KM, VAN, TPC><<<grid, KM * TPC, sm, st>>>(a);
@@ -292,7 +317,14 @@ static cudaError_t launch_small_cfg(const DenseArgs& a, int jobs, int resident, 
 
 template <int KM>
 static cudaError_t launch_small_class(const DenseArgs& a, int jobs, cudaStream_t st) {
-  const size_t sm = small_stage_logB<KM>(a) ? (size_t)a.V * KM * sizeof(float) : 0;
+  const size_t sm = small_smem<KM>(a);
+  if (sm > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(small_fwd_kernel<KM, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sm);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(small_fwd_kernel<KM, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+  }
   if (a.kind == kJobVanilla) return launch_small_cfg<KM, true, 2>(a, jobs, small_resident<KM, true, 2>(sm), st);
   const int r2 = small_resident<KM, false, 2>(sm);
   if (jobs <= r2) return launch_small_cfg<KM, false, 2>(a, jobs, r2, st);
