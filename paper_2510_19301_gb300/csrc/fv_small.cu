@@ -55,8 +55,11 @@ constexpr int kSmallAhead = 4;  // emission scores loaded this many steps ahead
 // two threads cut config 1's FLASH decode by 12% and slowed a 512-sequence
 // K=64 FLASH batch by 45%).
 // VAN: the exact-decoding instance (no MidState, snapshots or task lists,
-// fewer registers); otherwise every job kind of the engines
-template <int KM, bool VAN, int TPC>
+// fewer registers); otherwise every job kind of the engines.  DIRECT: leaf
+// tasks whose rows stay in shared memory; an instance of its own, since its
+// code in the common one slowed the other kinds (FLASH with a budget, K = 32
+// .. 80: by 2 to 12%)
+template <int KM, bool VAN, int TPC, bool DIRECT>
 __global__ void __launch_bounds__(KM * TPC, VAN ? (KM <= 64 ? 6 : 2) : (KM <= 64 ? 8 / TPC : 1)) small_fwd_kernel(DenseArgs a) {
   constexpr int RH = KM / TPC;  // rows per thread
   constexpr int Q = RH / 4;                      // rows per chain
@@ -109,7 +112,7 @@ __global__ void __launch_bounds__(KM * TPC, VAN ? (KM <= 64 ? 6 : 2) : (KM <= 64
     const Job jb = a.jobs[b];
     const int T = jb.T;
     if (T < 1 || n < m) return;
-    if (!VAN && a.direct && n - m > a.direct) {
+    if (DIRECT && n - m > a.direct) {
       // the lengths on the device are not the host's: no room for the rows
       if (tid == 0) set_status(a.hdr, FV_EINVAL, (uint32_t)b);
       return;
@@ -197,7 +200,7 @@ __global__ void __launch_bounds__(KM * TPC, VAN ? (KM <= 64 ? 6 : 2) : (KM <= 64
           if (other) { bv = ov; g = og; }
         }
         dval = own ? __fadd_rn(bv, e) : -CUDART_INF_F;
-        if (!VAN && a.direct) {
+        if (DIRECT) {
           if (lead) spsi[(t - m - 1) * KM + j] = (uint8_t)g;
         } else if (lead && own && (kind == kJobVanilla || kind == kJobLeaf)) {
           const int64_t row = kind == kJobVanilla ? jb.aux_off + (int64_t)t * K
@@ -252,7 +255,7 @@ __global__ void __launch_bounds__(KM * TPC, VAN ? (KM <= 64 ? 6 : 2) : (KM <= 64
         a.qlast[b] = qi;
         a.scores[b] = sd[cur][qi];
       }
-    } else if (!VAN && a.direct && tid == 0) {
+    } else if (DIRECT && tid == 0) {
       // q_{t-1} = psi_t[q_t] from the known q_n (the last step's barrier
       // completed the rows; the next job starts behind a barrier)
       int32_t* path = a.paths + jb.path_off;
@@ -294,10 +297,10 @@ static size_t small_smem(const DenseArgs& a) {
 // exact decoding: one CTA per sequence; other kinds: a persistent grid of
 // the CTAs resident at once (per instance), at most one per job
 // CTAs of the instance resident at once on the device (0 on an error)
-template <int KM, bool VAN, int TPC>
+template <int KM, bool VAN, int TPC, bool DIRECT>
 static int small_resident(size_t sm) {
   int per_sm = 0, dev = 0, nsm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, small_fwd_kernel<KM, VAN, TPC>, KM * TPC, sm) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, small_fwd_kernel<KM, VAN, TPC, DIRECT>, KM * TPC, sm) !=
           cudaSuccess ||
       cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
     cudaGetLastError();
@@ -306,29 +309,35 @@ static int small_resident(size_t sm) {
   return per_sm * nsm;
 }
 
-template <int KM, bool VAN, int TPC>
-static cudaError_t launch_small_cfg(const DenseArgs& a, int jobs, int resident, cudaStream_t st) {
-  const size_t sm = small_smem<KM>(a);
+template <int KM, bool VAN, int TPC, bool DIRECT>
+static cudaError_t launch_small_cfg(const DenseArgs& a, int jobs, int resident, size_t sm, cudaStream_t st) {
   if (resident < 1) return cudaErrorInvalidConfiguration;
   const int grid = VAN ? jobs : (jobs < resident ? jobs : resident);
-  small_fwd_kernel<KM, VAN, TPC><<<grid, KM * TPC, sm, st>>>(a);
+  small_fwd_kernel<KM, VAN, TPC, DIRECT><<<grid, KM * TPC, sm, st>>>(a);
   return cudaGetLastError();
+}
+
+template <int KM, bool DIRECT>
+static cudaError_t launch_small_tasks(const DenseArgs& a, int jobs, size_t sm, cudaStream_t st) {
+  if (sm > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(small_fwd_kernel<KM, false, 1, DIRECT>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(small_fwd_kernel<KM, false, 2, DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)sm);
+    if (e != cudaSuccess) return e;
+  }
+  const int r2 = small_resident<KM, false, 2, DIRECT>(sm);
+  if (jobs <= r2) return launch_small_cfg<KM, false, 2, DIRECT>(a, jobs, r2, sm, st);
+  return launch_small_cfg<KM, false, 1, DIRECT>(a, jobs, small_resident<KM, false, 1, DIRECT>(sm), sm, st);
 }
 
 template <int KM>
 static cudaError_t launch_small_class(const DenseArgs& a, int jobs, cudaStream_t st) {
   const size_t sm = small_smem<KM>(a);
-  if (sm > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(small_fwd_kernel<KM, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sm);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(small_fwd_kernel<KM, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-  }
-  if (a.kind == kJobVanilla) return launch_small_cfg<KM, true, 2>(a, jobs, small_resident<KM, true, 2>(sm), st);
-  const int r2 = small_resident<KM, false, 2>(sm);
-  if (jobs <= r2) return launch_small_cfg<KM, false, 2>(a, jobs, r2, st);
-  return launch_small_cfg<KM, false, 1>(a, jobs, small_resident<KM, false, 1>(sm), st);
+  if (a.kind == kJobVanilla)
+    return launch_small_cfg<KM, true, 2, false>(a, jobs, small_resident<KM, true, 2, false>(sm), sm, st);
+  return a.direct ? launch_small_tasks<KM, true>(a, jobs, sm, st) : launch_small_tasks<KM, false>(a, jobs, sm, st);
 }
 
 cudaError_t launch_small_forward(const DenseArgs& a, cudaStream_t st) {
