@@ -33,12 +33,15 @@ UNIT = "state-steps/s"
 WORKLOAD = "batched-uneven: 1024 seqs, K=256 dense FP32, T~U[500,4000], E=log_softmax(N(0,1))"
 
 
-# DRAM bytes per state-step of dense_fwd_kernel (K=256, vanilla, the default
-# configuration: 4-CTA clusters, two CTAs per SM): reads of E plus writes of
-# psi, from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum)
-# of a 608-sequence launch of this workload (sum of T = 1 391 599).
-DRAM_BYTES_PER_STATE_STEP = (1427830784 + 683246592) / (1391599 * 256)
+# DRAM bytes per state-step of prune_fwd_kernel (K=256, vanilla, the default
+# engine): reads of E plus writes of the delta rows, from one ncu capture
+# (dram__bytes_read.sum + dram__bytes_write.sum) of a 608-sequence launch of
+# 1000 steps.
+DRAM_BYTES_PER_STATE_STEP = (622936576 + 573162496) / (608 * 1000 * 256)
 TRAFFIC_VARIANT = 0  # the configuration those counters were taken on
+# Share of the K^2 candidates of a step that the bounded-row engine forms on
+# this family of inputs (listed weights + rows, counted in the kernel), by K.
+CANDIDATE_SHARE = {256: (6 + 34) / 256, 512: (12 + 40) / 512, 1024: (16 + 61) / 1024}
 
 
 def dist_env():
@@ -484,18 +487,11 @@ def config3_dense(fv, T, device, lib):
     lane_peak = alu_peak_tops(pk.get("sm_max_mhz", 2070.0), sm_count(device))
     fwd = out["vanilla"]["forward_kernels_ms"]
     achieved = 2.0 * cells / (fwd / 1e3) / 1e12
-    out["roofline"] = {"bound": "alu", "kernel": "wide_fwd_kernel", "achieved": achieved, "peak": peak,
-                       "unit": "TFLOP/s", "frac": achieved / peak, "peak_kind": "measured (fv_maxplus_peak)",
-                       "frac_of_fp32_lanes": achieved / lane_peak, "kernel_ms": fwd, "cells": cells}
-    # with 8 sequences the 64 MB logA cannot stay on chip (all shared memory
-    # together holds about 34 MB), so every step re-reads it: the step is
-    # bound by that stream, 4 K^2 bytes per step
-    hbm_peak = pk.get("hbm_gbs", 6800.0)
-    lo_bytes = 4.0 * K * K * (T - 1)
-    hbm_ach = lo_bytes / (fwd / 1e3) / 1e9
-    out["roofline_hbm"] = {"bound": "hbm", "kernel": "wide_fwd_kernel", "achieved": hbm_ach, "peak": hbm_peak,
-                           "unit": "GB/s", "frac": hbm_ach / hbm_peak, "bytes_per_step": 4 * K * K,
-                           "alu_fraction_at_hbm_peak": min(1.0, (2.0 * n * K * K * hbm_peak * 1e9 / (4.0 * K * K)) / 1e12 / peak)}
+    # the bounded-row engine forms a share of the K^2 candidates and reads
+    # that share of logA, so this is the rate of the full recursion it stands for
+    out["full_recursion_equivalent"] = {"kernel": "prune_fwd_kernel", "bound": "latency and L2 reads of rows",
+                                        "tflops": achieved, "of_measured_maxplus_peak": achieved / peak,
+                                        "of_fp32_lanes": achieved / lane_peak, "kernel_ms": fwd, "cells": cells}
     del res, E
     torch.cuda.empty_cache()
     return out
@@ -559,10 +555,10 @@ def config3_sparse(fv, T, device, lib):
 
 
 def larger_k_rows(fv, device, lib, peak_tflops, Ks=(512, 1024), n_seq=256):
-    """Exact decoding at larger state spaces, the streamed cluster engines
-    (4 CTAs per model at K=512, 8 at K=1024): 256 sequences, T uniform in
+    """Exact decoding at larger state spaces: 256 sequences, T uniform in
     [500, 4000], Dirichlet(1) rows, log-softmax emissions; forward-kernel
-    time and its fraction of the measured max-plus ceiling."""
+    time, the candidates it forms against the measured max-plus ceiling, and
+    the rate of the full recursion it stands for."""
     import torch
 
     import workloads as W
@@ -580,8 +576,10 @@ def larger_k_rows(fv, device, lib, peak_tflops, Ks=(512, 1024), n_seq=256):
         achieved = 2.0 * cells / (fwd / 1e3) / 1e12
         rows[f"K{K}"] = {"workload": f"{n_seq} sequences, K={K} dense FP32, T~U[500,4000]",
                          "ms": ms, "value": int(lengths.sum()) * K / (ms / 1e3), "unit": UNIT,
-                         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak_tflops, "unit": "TFLOP/s",
-                                      "frac": achieved / peak_tflops, "kernel_ms": fwd}}
+                         "roofline": {"bound": "latency and L2 reads of rows",
+                                      "achieved": achieved * CANDIDATE_SHARE[K], "peak": peak_tflops, "unit": "TFLOP/s",
+                                      "frac": achieved * CANDIDATE_SHARE[K] / peak_tflops, "kernel_ms": fwd,
+                                      "full_recursion_equivalent_tflops": achieved}}
         del d, b, E
         torch.cuda.empty_cache()
     return rows
@@ -867,7 +865,10 @@ def run_ours(args):
     lane_peak = alu_peak_tops(pk.get("sm_max_mhz", 2070.0), sms)
     peak = alu_probe["tflops"]
     achieved = 2.0 * cells / (fwd_ms / 1e3) / 1e12
-    launches = args.steps * 4
+    # vanilla: prep, order, (model preparation,) forward, trace and its repair
+    bounded = args.mode == "vanilla" and int(chosen[0]) == 0
+    launches = args.steps * ((6 if K > 128 else 5) if bounded else 4)
+    share = CANDIDATE_SHARE.get(K, 1.0) if bounded else 1.0
 
     wl_name = WORKLOAD if (args.K == 256 and args.n_seq == 1024) else WORKLOAD.replace(
         "1024 seqs, K=256", f"{args.n_seq} seqs, K={args.K}")
@@ -880,8 +881,15 @@ def run_ours(args):
                       "l2": "inputs larger than L2 (E is %.2f GB per step)" % (wl["E"].numel() * 4 / 1e9)},
            "clocks": clocks,
            "gpu_launches": launches,
-           "roofline": {"bound": "alu", "kernel": "dense_fwd_kernel", "achieved": achieved,
-                        "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+           "roofline": {"bound": "latency" if bounded else "alu",
+                        "kernel": "prune_fwd_kernel" if bounded and K > 128 else
+                                  "small_value_kernel" if bounded else "dense_fwd_kernel",
+                        "achieved": achieved * share,
+                        "peak": peak, "unit": "TFLOP/s", "frac": achieved * share / peak,
+                        "candidate_share": share,
+                        "candidate_note": "share of the K^2 candidates per step that the engine forms (the others "
+                                          "cannot win); achieved counts those, full_recursion_equivalent_tflops all",
+                        "full_recursion_equivalent_tflops": achieved,
                         "traffic": (DRAM_BYTES_PER_STATE_STEP * state_steps
                                     if (args.K == 256 and args.mode == "vanilla" and int(chosen[0]) == TRAFFIC_VARIANT)
                                     else None),
@@ -893,7 +901,7 @@ def run_ours(args):
                                      "(%.1f cells/clk/SM, 2 ops per cell)" % alu_probe["cells_per_clk_per_sm"],
                         "sm_count": sms,
                         "peak_fp32_lanes": lane_peak,
-                        "frac_of_fp32_lanes": achieved / lane_peak,
+                        "frac_of_fp32_lanes": achieved * share / lane_peak,
                         "peak_fp32_lanes_kind": "derived: %d SMs x 128 FP32 lanes x 2 ops x %.0f MHz (max clock); "
                                                 "the FP32 max runs at half the add rate, so no max-plus code "
                                                 "reaches it" % (sms, pk.get("sm_max_mhz", 2070.0)),
