@@ -247,6 +247,7 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M, BEAM>::NT, 1) p
   // barrier of the job's warps here; true where any thread passes true
   auto group_any = [&](bool x) -> bool {
     if constexpr (W == 1) {
+      __syncwarp();  // (a vote alone orders no memory between the lanes)
       return __any_sync(0xffffffffu, x);
     } else {
       uint32_t r;
