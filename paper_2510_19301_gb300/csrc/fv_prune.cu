@@ -208,7 +208,13 @@ struct PruneCfg {
   static constexpr bool COOP = W > 1 && (NW > 8 || BEAM);
   static constexpr int NL = KP + U;  // entries of a common list
   static constexpr size_t s_bytes = COOP ? (size_t)G * 2 * NL * 8 : 0;
-  static constexpr size_t smem = a_bytes + d_bytes + l_bytes + s_bytes;
+  // STAGE: the columns that the bulk copies send, double buffered.  A beam
+  // masks its delta at the start of the next step, when a copy may still be
+  // reading; without a beam the copies read delta itself, which is written
+  // again two steps later, once every CTA has the copy.
+  static constexpr bool STAGE = BEAM && CL > 2;
+  static constexpr size_t x_bytes = STAGE ? (size_t)2 * KH * 4 : 0;
+  static constexpr size_t smem = a_bytes + d_bytes + l_bytes + s_bytes + x_bytes;
 };
 // bounded wait of the cluster exchange (~1 s at 2 GHz)
 constexpr long long kPruneWaitCycles = 1ll << 31;
@@ -826,14 +832,22 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M, BEAM>::NT, 1) p
           }
         } else {
           // one copy of the CTA's columns to each of the others
+          const float* own = sd + cur * KP + (int)rank * KH;
+          if constexpr (Cfg::STAGE) {
+            float* sx = reinterpret_cast<float*>(smem + Cfg::a_bytes + Cfg::d_bytes + Cfg::l_bytes + Cfg::s_bytes) +
+                        cur * KH;
+#pragma unroll
+            for (int c = 0; c < C; ++c) sx[gt * C + c] = dval[c];
+            own = sx;
+          }
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           group_any(false);
           if (gt < CL && gt != (int)rank) {
-            const uint32_t src = smem_addr(sd + cur * KP + (int)rank * KH);
+            const uint32_t src = smem_addr(own), dst = smem_addr(sd + cur * KP + (int)rank * KH);
             const uint32_t to = dsmem_addr(smem, gt);
             asm volatile(
                 "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                    to + (src - self)),
+                    to + (dst - self)),
                 "r"(src), "r"(KH * 4), "r"(to + (bar - self))
                 : "memory");
           }
