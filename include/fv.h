@@ -183,14 +183,24 @@ typedef struct {
   uint32_t flags;
 } fv_params;
 
-/* Bytes of device workspace fv_decode needs for this request (>= 4096).
- * Returns 0 on invalid arguments. */
+/* Bytes of device workspace to give fv_decode for this request (>= 4096).
+ * Where decoding is faster with more than it needs (delta rows of 4 bytes per
+ * state-step in place of 2-byte backpointers for FV_VANILLA, row copies for
+ * FV_BEAM), this is the larger size, unless it exceeds half of the device's
+ * memory.  Returns 0 on invalid arguments. */
 size_t fv_workspace_size(const fv_model* models, int32_t n_models,
                          const fv_batch* batch, const fv_params* params);
 
+/* Bytes of the smallest workspace fv_decode takes for this request: at most
+ * fv_workspace_size, and about half of it for large FV_VANILLA batches.  The
+ * results are the same.  For callers that cannot spare the larger size.
+ * Returns 0 on invalid arguments. */
+size_t fv_workspace_min_size(const fv_model* models, int32_t n_models,
+                             const fv_batch* batch, const fv_params* params);
+
 /* Decode every sequence of the batch.  Writes paths_out (int32 state ids)
  * and scores_out[b] (the path's log-likelihood, forward order).  The
- * workspace must be 256-byte aligned and at least fv_workspace_size bytes;
+ * workspace must be 256-byte aligned and at least fv_workspace_min_size bytes;
  * its contents on entry do not matter.  Asynchronous on `stream`. */
 fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* batch,
                     const fv_params* params, void* workspace, size_t ws_bytes,

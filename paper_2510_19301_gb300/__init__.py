@@ -19,7 +19,7 @@ import torch
 from . import _lib as L
 from ._lib import FVError
 
-__all__ = ["Model", "Batch", "Decoder", "decode", "path_score", "workspace_size", "backward",
+__all__ = ["Model", "Batch", "Decoder", "decode", "path_score", "workspace_size", "workspace_min_size", "backward",
            "ViterbiScore", "FVError", "MODES", "autotune", "set_engine_variant"]
 
 MODES = {"vanilla": L.FV_VANILLA, "flash": L.FV_FLASH, "beam": L.FV_BEAM, "checkpoint": L.FV_CHECKPOINT}
@@ -163,6 +163,17 @@ def workspace_size(models, batch, mode="vanilla", P=1, B=0, mem_budget=0, flags=
     return int(lib.fv_workspace_size(arr, len(models), ctypes.byref(bs), ctypes.byref(ps)))
 
 
+def workspace_min_size(models, batch, mode="vanilla", P=1, B=0, mem_budget=0, flags=0):
+    """Bytes of the smallest workspace the request decodes in (the same
+    results; full-table decoding then keeps 2-byte backpointers in place of
+    4-byte delta rows, and runs slower)."""
+    lib = L.load()
+    arr = _models_array(models)
+    bs = batch.struct()
+    ps = _params(mode, P, B, mem_budget, flags)
+    return int(lib.fv_workspace_min_size(arr, len(models), ctypes.byref(bs), ctypes.byref(ps)))
+
+
 class Decoder:
     """A prepared decode call: structs, workspace and outputs are built once
     so that repeated launches cost one C call each (used by the benchmark)."""
@@ -180,8 +191,17 @@ class Decoder:
         if self.ws_bytes == 0:
             raise FVError(L.FV_EINVAL, "fv_workspace_size")
         dev = batch.device
-        self.workspace = workspace if workspace is not None else torch.empty(
-            self.ws_bytes, dtype=torch.uint8, device=dev)
+        if workspace is None:
+            try:
+                workspace = torch.empty(self.ws_bytes, dtype=torch.uint8, device=dev)
+            except torch.cuda.OutOfMemoryError:
+                small = int(self.lib.fv_workspace_min_size(self._arr, len(self.models), ctypes.byref(self._bs),
+                                                           ctypes.byref(self._ps)))
+                if not 0 < small < self.ws_bytes:
+                    raise
+                self.ws_bytes = small
+                workspace = torch.empty(small, dtype=torch.uint8, device=dev)
+        self.workspace = workspace
         if self.workspace.data_ptr() % 256:
             raise ValueError("workspace must be 256-byte aligned")
         self.paths = paths if paths is not None else torch.empty(max(batch.path_len, 1), dtype=torch.int32,

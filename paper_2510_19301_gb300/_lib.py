@@ -104,6 +104,8 @@ def load(build_if_missing: bool = False):
     MP, BP, PP = ctypes.POINTER(fv_model), ctypes.POINTER(fv_batch), ctypes.POINTER(fv_params)
     lib.fv_workspace_size.argtypes = [MP, i32, BP, PP]
     lib.fv_workspace_size.restype = sz
+    lib.fv_workspace_min_size.argtypes = [MP, i32, BP, PP]
+    lib.fv_workspace_min_size.restype = sz
     lib.fv_decode.argtypes = [MP, i32, BP, PP, P, sz, P, P, P]
     lib.fv_decode.restype = ctypes.c_int
     lib.fv_backward.argtypes = [MP, i32, BP, P, P, P, P, P, P, sz, P]

@@ -467,6 +467,17 @@ void timed_end(cudaStream_t st) {
   ++g_timed;
 }
 
+// below this, the device's memory is not asked for
+constexpr size_t kAskMemory = (size_t)8 << 30;
+size_t device_memory_bytes() {
+  size_t free_bytes = 0, total = 0;
+  if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return (size_t)284208 << 20;  // no device visible: GB300's
+  }
+  return total;
+}
+
 // Beam search (P = 0) and FLASH-BS (P >= 1) launch sequence, per model.
 fv_status decode_beam(const fv_model* models, int32_t n_models, const fv_batch* batch, const fv_params* p, char* ws,
                       const Layout& L, const FlashPlan& fp, const Ranges& R, int32_t* paths_out, float* scores_out,
@@ -663,8 +674,8 @@ fv_params exact_params(const fv_model* models, int32_t n_models, const fv_params
   return q;
 }
 
-size_t fv_workspace_size(const fv_model* models, int32_t n_models, const fv_batch* batch,
-                         const fv_params* p_in) {
+size_t fv_workspace_min_size(const fv_model* models, int32_t n_models, const fv_batch* batch,
+                             const fv_params* p_in) {
   if (!p_in || !batch || !batch->T_host) return 0;
   if (check_common(models, n_models, batch) != FV_OK) return 0;
   if (p_in->mode == FV_FLASH && p_in->P < 1) return 0;
@@ -678,19 +689,21 @@ size_t fv_workspace_size(const fv_model* models, int32_t n_models, const fv_batc
   }
   if (p->mode == FV_BEAM && p->B < 1) return 0;
   if (p->mode != FV_VANILLA && p->mode != FV_BEAM && p->mode != FV_CHECKPOINT) return 0;
-  const size_t base = layout_for(models, n_models, batch, p->mode, nullptr, p->B, p->P).total;
-  if (!delta_rows(models, n_models, p)) return base;
-  return std::max(base, layout_for(models, n_models, batch, p->mode, nullptr, p->B, 0, true).total);
+  return layout_for(models, n_models, batch, p->mode, nullptr, p->B, p->P).total;
 }
 
-}  // extern "C"
-
-size_t fv::exact_min_workspace(const fv_model* models, int32_t n_models, const fv_batch* batch) {
-  if (!batch || !batch->T_host || check_common(models, n_models, batch) != FV_OK) return 0;
-  return layout_for(models, n_models, batch, FV_VANILLA, nullptr).total;
+size_t fv_workspace_size(const fv_model* models, int32_t n_models, const fv_batch* batch,
+                         const fv_params* p_in) {
+  const size_t base = fv_workspace_min_size(models, n_models, batch, p_in);
+  if (!base) return 0;
+  const fv_params p = exact_params(models, n_models, p_in);
+  if (!delta_rows(models, n_models, &p)) return base;
+  const size_t rows = layout_for(models, n_models, batch, p.mode, nullptr, p.B, 0, true).total;
+  // Dense emission scores take as many bytes as the delta rows: beyond half
+  // of the device's memory the two do not fit, where the smaller table may.
+  if (rows > kAskMemory && rows > device_memory_bytes() / 2) return base;
+  return std::max(base, rows);
 }
-
-extern "C" {
 
 fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* batch, const fv_params* p_in,
                     void* workspace, size_t ws_bytes, int32_t* paths_out, float* scores_out,

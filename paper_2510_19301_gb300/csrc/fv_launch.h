@@ -223,10 +223,6 @@ struct ScoreArgs {
   const int32_t* obs;
 };
 
-// Smallest workspace that exact decoding of dense models runs in (psi rows;
-// fv_workspace_size asks for delta rows where the bounded-row engine decodes).
-size_t exact_min_workspace(const fv_model* models, int32_t n_models, const fv_batch* batch);
-
 int dense_supported_K(int K);
 // Engine configuration variants of a K class and the tuned choice.
 int dense_k_class(int K);

@@ -16,7 +16,6 @@
 #include <mutex>
 
 #include "../../include/fv.h"
-#include "fv_launch.h"
 
 namespace {
 
@@ -67,7 +66,7 @@ extern "C" fv_status fv_decode_noalloc(const fv_model* models, int32_t n_models,
   p.B = 0;
   p.mem_budget_bytes = 0;
   p.flags = 0;
-  const size_t need = fv::exact_min_workspace(models, n_models, batch);
+  const size_t need = fv_workspace_min_size(models, n_models, batch, &p);
   if (need == 0) return FV_EINVAL;
   if (need > kScratchBytes) return FV_ENOMEM;  // request larger than the static scratch
   void* ws = nullptr;
