@@ -57,6 +57,7 @@ class Request:
     finished: float = math.nan
     status: int = -1
     nbytes: int = 0
+    compact: bool = False        # decode in the smallest workspace (full-table requests too large otherwise)
     result: object = None
 
     @property
@@ -66,7 +67,8 @@ class Request:
     @property
     def klass(self):
         """Requests of one class can share one launch."""
-        return (self.K, self.mode, self.B if self.mode == "beam" else 0, self.P if self.mode != "exact" else 0)
+        return (self.K, self.mode, self.B if self.mode == "beam" else 0, self.P if self.mode != "exact" else 0,
+                self.compact)
 
 
 class Server:
@@ -126,6 +128,9 @@ class Server:
         while self.waiting:
             req = self.waiting[0]
             need = self.backend.bytes_needed(req)
+            if need > self.budget and not req.compact:
+                req.compact = True
+                need = self.backend.bytes_needed(req)
             if need > self.budget:  # can never fit: reject instead of blocking the queue
                 self.waiting.popleft()
                 self._fail(req, -2)
@@ -218,10 +223,11 @@ class GpuBackend:
                  shared_models: bool = True, model_seed: int = 6):
         import torch
 
-        from . import Batch, Decoder, Model
+        from . import Batch, Decoder, Model, workspace_min_size
         from ._lib import FV_SHARED_GPU
         self.torch = torch
         self.Batch, self.Decoder, self.Model = Batch, Decoder, Model
+        self.workspace_min_size = workspace_min_size
         self.FV_SHARED_GPU = FV_SHARED_GPU
         self.device = device
         self.streams = [torch.cuda.Stream(device=device) for _ in range(n_streams)]
@@ -292,7 +298,7 @@ class GpuBackend:
         inputs = 4 * (T * K) + (0 if self.shared else 4 * (K * K + K))
         outputs = 4 * (T + 1)
         if req.mode == "exact":
-            ws = 2 * T * K
+            ws = (2 if req.compact else 4) * T * K  # backpointers or delta rows
         elif req.mode == "beam":
             ws = 8 * T * min(req.B, K) + 4 * 4 * K
         else:
@@ -324,8 +330,12 @@ class GpuBackend:
             mi = list(range(len(reqs)))
         b = self.Batch(lengths, E=E, models=models, model_index=mi, device=self.device)
         # launches overlap on the device: kernels with the least SM time per step
-        dec = self.Decoder(models, b, mode=self._mode(r0), P=r0.P if r0.mode != "exact" else 1,
-                           B=r0.B if r0.mode == "beam" else 0, flags=self.FV_SHARED_GPU)
+        how = dict(mode=self._mode(r0), P=r0.P if r0.mode != "exact" else 1, B=r0.B if r0.mode == "beam" else 0,
+                   flags=self.FV_SHARED_GPU)
+        ws = None
+        if r0.compact:
+            ws = torch.empty(self.workspace_min_size(models, b, **how), dtype=torch.uint8, device=self.device)
+        dec = self.Decoder(models, b, workspace=ws, **how)
         return dec, E, models
 
     def launch_batch(self, reqs):
