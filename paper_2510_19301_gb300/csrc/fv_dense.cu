@@ -1456,7 +1456,7 @@ int dense_get_variant(int K) { return g_variant[dense_k_class(K)]; }
 // 160 rows of at most 128 bytes: 20 KB next to the staged symbol table, so the
 // one-CTA-per-job engine keeps its two CTAs (K = 128) per SM
 int dense_direct_rows(int K, bool no_tune) {
-  return K <= 128 && (no_tune || g_variant[dense_k_class(K)] == 0) ? 160 : 0;
+  return K <= 128 && (no_tune || g_variant[dense_k_class(K)] == 0) ? kDirectRows : 0;
 }
 bool dense_prune_K(int K) { return K <= 4096; }
 bool dense_uses_prune(int K, bool no_tune, bool withhold) {

@@ -250,6 +250,7 @@ bool prune_beam_wins(int K, int64_t sum_T, int max_T, bool alone);
 cudaError_t launch_prune_beam(const DenseArgs& a, bool alone, cudaStream_t st);
 // FLASH tasks of at most this many backpointer rows are solved in one launch
 // (K <= 128 on the default engine; 0: not there)
+constexpr int kDirectRows = 160;
 int dense_direct_rows(int K, bool no_tune);
 bool dense_prune_K(int K);
 bool dense_uses_prune(int K, bool no_tune, bool withhold);

@@ -27,6 +27,8 @@
 #include <math_constants.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "fv_internal.cuh"
 #include "fv_launch.h"
 
@@ -294,15 +296,32 @@ static size_t small_smem(const DenseArgs& a) {
   return (small_stage_logB<KM>(a) ? (size_t)a.V * KM * sizeof(float) : 0) + (size_t)a.direct * KM;
 }
 
+// Dynamic shared memory beyond 48 KB less the kernel's static shared memory
+// has to be allowed first.  The limit is state of the process, so each
+// instance gets the largest size that any call can need, once per device: no
+// call's size is left to what other calls, or other threads, have set.
+template <int KM, bool VAN, int TPC, bool DIRECT>
+static bool small_allow_smem(int dev) {
+  static std::atomic<bool> done[64];
+  const bool known = dev >= 0 && dev < 64;
+  if (known && done[dev].load()) return true;
+  if (cudaFuncSetAttribute(small_fwd_kernel<KM, VAN, TPC, DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           kSmallLogB + (DIRECT ? kDirectRows * KM : 0)) != cudaSuccess)
+    return false;
+  if (known) done[dev].store(true);
+  return true;
+}
+
 // exact decoding: one CTA per sequence; other kinds: a persistent grid of
 // the CTAs resident at once (per instance), at most one per job
 // CTAs of the instance resident at once on the device (0 on an error)
 template <int KM, bool VAN, int TPC, bool DIRECT>
 static int small_resident(size_t sm) {
   int per_sm = 0, dev = 0, nsm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, small_fwd_kernel<KM, VAN, TPC, DIRECT>, KM * TPC, sm) !=
+  if (cudaGetDevice(&dev) != cudaSuccess || !small_allow_smem<KM, VAN, TPC, DIRECT>(dev) ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, small_fwd_kernel<KM, VAN, TPC, DIRECT>, KM * TPC, sm) !=
           cudaSuccess ||
-      cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -319,14 +338,6 @@ static cudaError_t launch_small_cfg(const DenseArgs& a, int jobs, int resident, 
 
 template <int KM, bool DIRECT>
 static cudaError_t launch_small_tasks(const DenseArgs& a, int jobs, size_t sm, cudaStream_t st) {
-  if (sm > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(small_fwd_kernel<KM, false, 1, DIRECT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(small_fwd_kernel<KM, false, 2, DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)sm);
-    if (e != cudaSuccess) return e;
-  }
   const int r2 = small_resident<KM, false, 2, DIRECT>(sm);
   if (jobs <= r2) return launch_small_cfg<KM, false, 2, DIRECT>(a, jobs, r2, sm, st);
   return launch_small_cfg<KM, false, 1, DIRECT>(a, jobs, small_resident<KM, false, 1, DIRECT>(sm), sm, st);
