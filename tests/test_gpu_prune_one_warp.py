@@ -24,7 +24,7 @@ def test_every_sequence_equals_the_backpointer_engines(K, n, T):
     E = torch.log_softmax(torch.randn(int(lengths.sum()), K, generator=g, device="cuda"), dim=-1)
     b = fv.Batch(lengths, E=E, models=[m])
     dec = fv.Decoder([m], b)
-    small = fv.Decoder([m], b, workspace=torch.empty(dec.ws_bytes * 3 // 4, dtype=torch.uint8, device="cuda"))
+    small = fv.Decoder([m], b, workspace=torch.empty(fv.workspace_min_size([m], b), dtype=torch.uint8, device="cuda"))
     p, s = (x.clone() for x in small())
     for _ in range(3):
         dec.paths.fill_(-1)
