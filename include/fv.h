@@ -95,9 +95,11 @@ typedef enum { FV_EMIT_DENSE = 0, FV_EMIT_DISCRETE = 1 } fv_emit_kind;
  * Results are the same either way. */
 #define FV_SHARED_GPU 0x20u
 /* Test hook for failure detection: the first CTA of the whole-GPU engine
- * (dense K > 1024) never publishes its step count, and CTA 1 of every 4- or
+ * (dense K > 1024) never publishes its step count, CTA 1 of every 4- or
  * 8-CTA cluster of the streamed engine (256 < K <= 1024) withholds its
- * arrivals on the delta exchange of the second tick, so the bounded waits on
+ * arrivals on the delta exchange of the second tick, and CTA 1 of every
+ * cluster of the bounded-row engine (128 < K <= 4096, exact decoding and
+ * dynamic beams) its delta of the second step, so the bounded waits on
  * them run out (about one second each); the call then reports FV_ETIMEOUT in
  * the status word and the CUDA context stays usable.  No other effect. */
 #define FV_TEST_WITHHOLD_STEP 0x80000000u

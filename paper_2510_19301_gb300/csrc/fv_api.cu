@@ -549,6 +549,7 @@ fv_status decode_beam(const fv_model* models, int32_t n_models, const fv_batch* 
       da.qlast = qlast;
       da.scores = scores_out;
       da.hdr = hdr;
+      da.wide_withhold = (p->flags & FV_TEST_WITHHOLD_STEP) ? 1 : 0;
       da.beam_B = p->B;
       da.beam_stride = L.Wcap;
       da.beam_id = reinterpret_cast<int32_t*>(ws + L.aux);
@@ -738,7 +739,7 @@ fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* ba
   bool prune = batch->T_host && n > 0 && delta_rows(models, n_models, p);
   for (int m = 0; m < n_models && prune; ++m)
     prune = p->mode == FV_BEAM ||
-            dense_uses_prune(models[m].K, (p->flags & FV_NO_TUNE) != 0, (p->flags & FV_TEST_WITHHOLD_STEP) != 0);
+            dense_uses_prune(models[m].K, (p->flags & FV_NO_TUNE) != 0);
   // (preparing a model above K = 2048 costs more than the whole-GPU engine's
   // steps up to about 30: K = 4096, 5 / 20 steps 326 / 497 against 210 / 482 us)
   if (prune && p->mode == FV_VANILLA) {

@@ -1459,8 +1459,8 @@ int dense_direct_rows(int K, bool no_tune) {
   return K <= 128 && (no_tune || g_variant[dense_k_class(K)] == 0) ? kDirectRows : 0;
 }
 bool dense_prune_K(int K) { return K <= 4096; }
-bool dense_uses_prune(int K, bool no_tune, bool withhold) {
-  return dense_prune_K(K) && !withhold && (no_tune || g_variant[dense_k_class(K)] == 0);
+bool dense_uses_prune(int K, bool no_tune) {
+  return dense_prune_K(K) && (no_tune || g_variant[dense_k_class(K)] == 0);
 }
 
 cudaError_t launch_dense_forward(DenseArgs a, int max_clusters, cudaStream_t st) {

@@ -128,7 +128,8 @@ struct DenseArgs {
   const float* wide_AT;       // column-major copy of logA, AT[j * wide_lane_stride(K) + i] = A[i][j]
                               // (streamed and whole-GPU configurations: the exact re-scan reads it)
   int32_t wide_withhold;      // test hook: CTA 0 of the whole-GPU engine never publishes its step count;
-                              // CTA 1 of each 4- / 8-CTA cluster withholds its second-tick arrivals
+                              // CTA 1 of each 4- / 8-CTA cluster withholds its second-tick arrivals, and
+                              // of each cluster of the bounded-row engine its second step's delta
   // bounded-row engine (fv_prune.cu; null: not prepared): padded row copy of
   // logA, per column the list of its largest weights, their rows, the cutoff
   const float* pr_A;
@@ -253,7 +254,7 @@ cudaError_t launch_prune_beam(const DenseArgs& a, bool alone, cudaStream_t st);
 constexpr int kDirectRows = 160;
 int dense_direct_rows(int K, bool no_tune);
 bool dense_prune_K(int K);
-bool dense_uses_prune(int K, bool no_tune, bool withhold);
+bool dense_uses_prune(int K, bool no_tune);
 // exact decoding at K <= 128, values only: delta rows to a.pr_D (fv_small.cu)
 cudaError_t launch_small_values(const DenseArgs& a, cudaStream_t st);
 // AT[j * KD + i] = logA[i * K + j] (rows K..KD-1 are -inf), KD = wide_lane_stride(K).

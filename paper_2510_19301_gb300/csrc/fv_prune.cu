@@ -810,6 +810,8 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M, BEAM>::NT, 1) p
       else dn[0] = dval[0];
       if constexpr (CL > 1) {
         const uint32_t bar = smem_addr(&s_bar[grp][cur]);
+        // test hook: CTA 1 keeps its second step from the others
+        const bool withhold = t == 1 && rank == 1 && a.wide_withhold;
         if (gt == 0) mbar_arrive_expect_tx(bar, (CL - 1) * KH * 4);
         if constexpr (CL == 2) {
           // 16 bytes per store: four lanes' columns where a lane has one
@@ -825,7 +827,7 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M, BEAM>::NT, 1) p
             c4 = col0 - lane * C + 4 * (send ? lane : 0);
             v = *reinterpret_cast<const uint4*>(sd + cur * KP + c4);
           }
-          if (send) {
+          if (send && !withhold) {
             const uint32_t off = smem_addr(sd + cur * KP + c4) - self, boff = bar - self;
             const uint32_t to = rank ? peer[0] : peer[1];
             st_async_v4(to + off, v, to + boff);
@@ -842,7 +844,7 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M, BEAM>::NT, 1) p
           }
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           group_any(false);
-          if (gt < CL && gt != (int)rank) {
+          if (gt < CL && gt != (int)rank && !withhold) {
             const uint32_t src = smem_addr(own), dst = smem_addr(sd + cur * KP + (int)rank * KH);
             const uint32_t to = dsmem_addr(smem, gt);
             asm volatile(
