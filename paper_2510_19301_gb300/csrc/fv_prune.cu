@@ -918,7 +918,22 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M, BEAM>::NT, 1) p
   if constexpr (CL > 1) {
     // no CTA leaves while another may still write to it or read its barriers
     __syncwarp();
+    if (!live && lane < CL) dsmem_st_u32(dsmem_addr(&s_stop[rank], lane), 1u);
+    __syncwarp();
     cluster_sync_all();
+    // where a wait ran out, a CTA may have left the steps before data that
+    // was sent to it arrived: every copy of the cluster is on its way by now
+    // and lands within the delay
+    bool any = false;
+#pragma unroll
+    for (int r = 0; r < CL; ++r) any |= s_stop[r] != 0;
+    if (any) {
+      const long long w0 = clock64();
+      while (clock64() - w0 < (1ll << 18)) {
+      }
+      __syncwarp();
+      cluster_sync_all();
+    }
   }
 }
 
