@@ -1095,32 +1095,36 @@ __global__ void __launch_bounds__(32 * TW) prune_trace_kernel(TraceArgs a) {
   if (a.hdr->status != 0) return;
   const int b = a.order[a.begin + blockIdx.x];
   const Job jb = a.jobs[b];
-  const int s = blockIdx.y, T = jb.T, K = a.K, lo = s * a.seg;
-  if (lo >= T) return;
+  const int T = jb.T, K = a.K;
   Tracer<VPL, TW, BEAM, ROWS> tr;
   tr.init(a, jb, part);
   int32_t* path = a.paths + jb.path_off;
   const bool lead = threadIdx.x == 0;
-  int q = a.qlast[b];
-  q = (unsigned)q < (unsigned)K ? q : 0;
-  int t = T - 1;  // q = q_t
-  if (T - lo > a.seg) {
-    const int hi = lo + a.seg;  // hi <= T - 1
-    if (hi + kTraceWarm < T - 1) {
-      t = hi + kTraceWarm;
-      q = tr.best(t);
+  // (a segment each, where the lengths here are no longer than the host's
+  // that sized the grid)
+  for (int64_t s = blockIdx.y; s * a.seg < T; s += gridDim.y) {
+    const int lo = (int)s * a.seg;
+    int q = a.qlast[b];
+    q = (unsigned)q < (unsigned)K ? q : 0;
+    int t = T - 1;  // q = q_t
+    if (T - lo > a.seg) {
+      const int hi = lo + a.seg;  // hi <= T - 1
+      if (hi + kTraceWarm < T - 1) {
+        t = hi + kTraceWarm;
+        q = tr.best(t);
+      }
+      q = tr.run(t, hi, q, [](int, int) { return false; });
+      t = hi;
+      const int64_t g = guess_off(a, jb, b) + s;
+      if (lead && g < a.guess_cap) a.guess[g] = q;
+    } else if (lead) {
+      path[t] = q;
     }
-    q = tr.run(t, hi, q, [](int, int) { return false; });
-    t = hi;
-    const int64_t g = guess_off(a, jb, b) + s;
-    if (lead && g < a.guess_cap) a.guess[g] = q;
-  } else if (lead) {
-    path[t] = q;
+    tr.run(t, lo, q, [&](int u, int x) {
+      if (lead) path[u] = x;
+      return false;
+    });
   }
-  tr.run(t, lo, q, [&](int u, int x) {
-    if (lead) path[u] = x;
-    return false;
-  });
 }
 
 template <int VPL, int TW, bool BEAM, bool ROWS>
@@ -1320,8 +1324,9 @@ size_t prune_guess_bytes(uint64_t aux_elems, int32_t n_seq, int64_t sum_T, int32
 }
 
 template <int VPL, int TW, bool BEAM, bool ROWS>
-static cudaError_t launch_trace_cfg(const TraceArgs& t, int max_T, cudaStream_t st) {
+static cudaError_t launch_trace_cfg(TraceArgs t, int max_T, cudaStream_t st) {
   const dim3 grid(t.count, (max_T + t.seg - 1) / t.seg);
+  if (grid.y == 1) t.seg = 0x7fffffff;  // one segment whatever the length on the device: no repair to launch
   prune_trace_kernel<VPL, TW, BEAM, ROWS><<<grid, 32 * TW, 0, st>>>(t);
   if (grid.y > 1) prune_fix_kernel<VPL, TW, BEAM, ROWS><<<t.count, 32 * TW, 0, st>>>(t);
   return cudaGetLastError();
