@@ -890,7 +890,13 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M, BEAM>::NT, 1) p
       }
     }
     if (!live) break;
-    if (BEAM && dead) break;
+    if (BEAM && dead) {
+      // the same in every CTA of the cluster, before anything of the step was
+      // exchanged; the next job clears what this one read
+      dead = false;
+      group_any(false);
+      continue;
+    }
     if (rank == 0 && gw == 0) {
       // termination: q_{T-1} = lowest argmax_j delta_{T-1}[j], score = delta_{T-1}[q]
       const float* dl = sd + ((ph - 1u) & 1u) * KP;
