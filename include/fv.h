@@ -256,25 +256,34 @@ fv_status fv_timing_pairs(float* ms, int32_t max_pairs, int32_t* n_pairs);
 
 /* Autotuning of the exact forward engine (not in the paper).  Dense exact
  * decoding has, per class of K (<= 64, <= 128, <= 256, <= 512, <= 1024),
- * several engine configurations -- the one-CTA-per-job small-K engine
- * (K <= 128), cluster sizes, CTAs per SM, warps per CTA and columns per
- * lane -- that compute the same values in the same order and differ only
- * in speed.  fv_autotune
- * decodes the given request once per candidate of every class present
- * (one warm-up and two timed calls each, CUDA events on `stream`), keeps
- * the fastest per class for every later fv_decode in this process, and
- * writes the chosen variant of each model's class to chosen[m] (may be
- * NULL).  Same arguments and outputs as fv_decode; it synchronises the
- * stream, so it is not capturable.  Requests without tunable classes
- * return FV_OK at once with chosen[] = 0.  Device errors are returned. */
+ * several engine configurations with the same results that differ only in
+ * speed.  Variant 0 is the default: for FV_VANILLA the engines that keep
+ * delta rows (K <= 128: values only; above: bounded candidate rows), for
+ * FV_FLASH and FV_CHECKPOINT, and for FV_VANILLA in the smallest workspace,
+ * the small-K engine (K <= 128) and the default cluster configuration; the
+ * others differ in cluster size, CTAs per SM, warps per CTA and columns per
+ * lane.  fv_autotune decodes the given request once per candidate of every
+ * class present (one warm-up and two timed calls each, CUDA events on
+ * `stream`), keeps the fastest per class for later fv_decode calls in this
+ * process, and writes the chosen variant of each model's class to chosen[m]
+ * (may be NULL).  A choice made for FV_FLASH or FV_CHECKPOINT holds for these
+ * two; one made for FV_VANILLA holds for all three, but FV_VANILLA keeps
+ * variant 0 where that is faster than the best of the others.  Same
+ * arguments and outputs as fv_decode; it synchronises the stream, so it is
+ * not capturable.  Requests without tunable classes return FV_OK at once
+ * with chosen[] = 0.  Device errors are returned. */
 fv_status fv_autotune(const fv_model* models, int32_t n_models, const fv_batch* batch,
                       const fv_params* params, void* workspace, size_t ws_bytes,
                       int32_t* paths_out, float* scores_out, fv_stream_t stream,
                       int32_t* chosen);
 
-/* Set the engine variant of K's class directly (0 = default); returns the
- * number of variants of that class.  For tuning studies and tests. */
+/* Set the engine variant of K's class directly, for every mode (0 =
+ * default); returns the number of variants of that class.  For tuning
+ * studies and tests. */
 int32_t fv_set_engine_variant(int32_t K, int32_t variant);
+
+/* The variant that fv_decode would use for K's class in a mode. */
+int32_t fv_get_engine_variant(int32_t K, int32_t mode);
 
 /* Bytes of the static device scratch behind fv_decode_noalloc. */
 #define FV_NOALLOC_SCRATCH_BYTES ((size_t)16 << 20)

@@ -20,7 +20,7 @@ from . import _lib as L
 from ._lib import FVError
 
 __all__ = ["Model", "Batch", "Decoder", "decode", "path_score", "workspace_size", "workspace_min_size", "backward",
-           "ViterbiScore", "FVError", "MODES", "autotune", "set_engine_variant"]
+           "ViterbiScore", "FVError", "MODES", "autotune", "set_engine_variant", "engine_variant"]
 
 MODES = {"vanilla": L.FV_VANILLA, "flash": L.FV_FLASH, "beam": L.FV_BEAM, "checkpoint": L.FV_CHECKPOINT}
 
@@ -232,8 +232,9 @@ class Decoder:
 
 def autotune(models, batch, mode="vanilla", P=1, B=0, mem_budget=0, flags=0, stream=None):
     """Time every engine configuration of the K classes in this request and
-    keep the fastest for later decodes in this process (fv_autotune).
-    Returns the chosen variant per model."""
+    keep the fastest for later decodes in this process (fv_autotune; a choice
+    made for "flash" or "checkpoint" does not touch "vanilla").  Returns the
+    chosen variant per model."""
     if isinstance(models, Model):
         models = [models]
     d = Decoder(models, batch, mode=mode, P=P, B=B, mem_budget=mem_budget, flags=flags)
@@ -248,9 +249,14 @@ def autotune(models, batch, mode="vanilla", P=1, B=0, mem_budget=0, flags=0, str
 
 
 def set_engine_variant(K, variant):
-    """Force the engine variant of K's class (0 = default); returns the
-    number of variants of that class."""
+    """Force the engine variant of K's class in every mode (0 = default);
+    returns the number of variants of that class."""
     return int(L.load().fv_set_engine_variant(int(K), int(variant)))
+
+
+def engine_variant(K, mode="vanilla"):
+    """The engine variant in use for K's class in a mode."""
+    return int(L.load().fv_get_engine_variant(int(K), MODES[mode]))
 
 
 def decode(models, batch, mode="vanilla", P=1, B=0, mem_budget=0, flags=0, stream=None, check=True):

@@ -134,6 +134,8 @@ def load(build_if_missing: bool = False):
     lib.fv_autotune.restype = ctypes.c_int
     lib.fv_set_engine_variant.argtypes = [i32, i32]
     lib.fv_set_engine_variant.restype = i32
+    lib.fv_get_engine_variant.argtypes = [i32, i32]
+    lib.fv_get_engine_variant.restype = i32
     lib.fv_maxplus_peak.argtypes = [i32, P, P, P, P]
     lib.fv_maxplus_peak.restype = ctypes.c_int
     lib.fv_version.argtypes = []

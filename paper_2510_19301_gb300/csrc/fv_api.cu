@@ -1100,8 +1100,13 @@ fv_status fv_backward(const fv_model* models, int32_t n_models, const fv_batch* 
 
 int32_t fv_set_engine_variant(int32_t K, int32_t variant) {
   if (K < 1) return 0;
-  dense_set_variant(K, variant);
+  dense_set_variant(K, true, variant);
+  dense_set_variant(K, false, variant);
   return dense_variants(K);
+}
+
+int32_t fv_get_engine_variant(int32_t K, int32_t mode) {
+  return K < 1 || mode == FV_BEAM ? 0 : dense_get_variant(K, mode == FV_VANILLA);
 }
 
 fv_status fv_autotune(const fv_model* models, int32_t n_models, const fv_batch* batch, const fv_params* p,
@@ -1126,32 +1131,47 @@ fv_status fv_autotune(const fv_model* models, int32_t n_models, const fv_batch* 
   run.flags &= ~FV_NO_TUNE;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (!reps.empty() && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)) return FV_ECUDA;
+  // two timed decodes of the request in `bytes` of the workspace
+  auto timed = [&](size_t bytes, float* ms) -> fv_status {
+    fv_status r = fv_decode(models, n_models, batch, &run, workspace, bytes, paths_out, scores_out, stream);
+    if (r != FV_OK) return r;
+    cudaEventRecord(e0, st);
+    for (int i = 0; i < 2 && r == FV_OK; ++i)
+      r = fv_decode(models, n_models, batch, &run, workspace, bytes, paths_out, scores_out, stream);
+    cudaEventRecord(e1, st);
+    if (r != FV_OK) return r;
+    if (cudaEventSynchronize(e1) != cudaSuccess) return FV_ECUDA;
+    cudaEventElapsedTime(ms, e0, e1);
+    return fv_last_device_status(workspace, stream);
+  };
+  // A full-table request finds the class's best engine with backpointer rows
+  // (in the workspace size where every variant is one), which FLASH and
+  // Checkpoint use too, and keeps it for itself only where it beats variant
+  // 0 in the whole workspace.  The other modes leave full-table decoding alone.
+  const bool table = q.mode == FV_VANILLA;
+  const size_t least = table ? std::min(ws_bytes, fv_workspace_min_size(models, n_models, batch, p)) : ws_bytes;
   for (int32_t K : reps) {
-    float best = 0.f;
+    float best = 0.f, ms = 0.f;
     int bv = 0;
     for (int v = 0; v < dense_variants(K); ++v) {
-      dense_set_variant(K, v);
-      s = fv_decode(models, n_models, batch, &run, workspace, ws_bytes, paths_out, scores_out, stream);
+      dense_set_variant(K, false, v);
+      if (table) dense_set_variant(K, true, v);
+      s = timed(least ? least : ws_bytes, &ms);
       if (s != FV_OK) break;
-      cudaEventRecord(e0, st);
-      for (int r = 0; r < 2 && s == FV_OK; ++r)
-        s = fv_decode(models, n_models, batch, &run, workspace, ws_bytes, paths_out, scores_out, stream);
-      cudaEventRecord(e1, st);
-      if (s != FV_OK) break;
-      if (cudaEventSynchronize(e1) != cudaSuccess) { s = FV_ECUDA; break; }
-      s = fv_last_device_status(workspace, stream);
-      if (s != FV_OK) break;
-      float ms = 0.f;
-      cudaEventElapsedTime(&ms, e0, e1);
       if (v == 0 || ms < best) { best = ms; bv = v; }
     }
-    dense_set_variant(K, s == FV_OK ? bv : 0);
+    if (s == FV_OK && table && bv != 0) {
+      dense_set_variant(K, true, 0);
+      s = timed(ws_bytes, &ms);
+    }
+    dense_set_variant(K, false, s == FV_OK ? bv : 0);
+    if (table) dense_set_variant(K, true, s == FV_OK && bv != 0 && best < ms ? bv : 0);
     if (s != FV_OK) break;
   }
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   if (chosen)
-    for (int m = 0; m < n_models; ++m) chosen[m] = q.mode == FV_BEAM ? 0 : dense_get_variant(models[m].K);
+    for (int m = 0; m < n_models; ++m) chosen[m] = fv_get_engine_variant(models[m].K, q.mode);
   return s;
 }
 

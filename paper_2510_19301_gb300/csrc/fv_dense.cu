@@ -1445,27 +1445,28 @@ int dense_variants(int K) {
   }
 }
 
-static int g_variant[6] = {0, 0, 0, 0, 0, 0};  // chosen by fv_autotune
+// chosen by fv_autotune, per class: for full-table decoding (0), whose
+// variant 0 is the bounded-row engine, and for FLASH and Checkpoint (1)
+static int g_variant[2][6];
 
-void dense_set_variant(int K, int v) {
-  const int c = dense_k_class(K);
-  g_variant[c] = (v >= 0 && v < dense_variants(K)) ? v : 0;
+void dense_set_variant(int K, bool table, int v) {
+  g_variant[table ? 0 : 1][dense_k_class(K)] = (v >= 0 && v < dense_variants(K)) ? v : 0;
 }
-int dense_get_variant(int K) { return g_variant[dense_k_class(K)]; }
+int dense_get_variant(int K, bool table) { return g_variant[table ? 0 : 1][dense_k_class(K)]; }
 
 // 160 rows of at most 128 bytes: 20 KB next to the staged symbol table, so the
 // one-CTA-per-job engine keeps its two CTAs (K = 128) per SM
 int dense_direct_rows(int K, bool no_tune) {
-  return K <= 128 && (no_tune || g_variant[dense_k_class(K)] == 0) ? kDirectRows : 0;
+  return K <= 128 && (no_tune || dense_get_variant(K, false) == 0) ? kDirectRows : 0;
 }
 bool dense_prune_K(int K) { return K <= 4096; }
 bool dense_uses_prune(int K, bool no_tune) {
-  return dense_prune_K(K) && (no_tune || g_variant[dense_k_class(K)] == 0);
+  return dense_prune_K(K) && (no_tune || dense_get_variant(K, true) == 0);
 }
 
 cudaError_t launch_dense_forward(DenseArgs a, int max_clusters, cudaStream_t st) {
   if (a.K > 1024) return launch_wide_forward(a, st);
-  const int v = a.no_tune ? 0 : g_variant[dense_k_class(a.K)];
+  const int v = a.no_tune ? 0 : dense_get_variant(a.K, a.kind == kJobVanilla);
   if (a.K <= 64) {
     if (v == 1) return launch_dense_cfg<64, 16, 8, 1, 64, false, 4>(a, max_clusters, st);
     if (v == 2) return launch_dense_cfg<64, 16, 16, 1, 64, false, 4>(a, max_clusters, st);

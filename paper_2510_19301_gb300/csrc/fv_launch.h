@@ -225,12 +225,13 @@ struct ScoreArgs {
 };
 
 int dense_supported_K(int K);
-// Engine configuration variants of a K class and the tuned choice.
+// Engine configuration variants of a K class and the tuned choice, for
+// full-table decoding (`table`) or for FLASH and Checkpoint.
 int dense_k_class(int K);
 int dense_job_slots(int K);
 int dense_variants(int K);
-void dense_set_variant(int K, int v);
-int dense_get_variant(int K);
+void dense_set_variant(int K, bool table, int v);
+int dense_get_variant(int K, bool table);
 int device_sm_count();
 bool wide_geometry(int K, int nsm, WideGeom* g);
 size_t wide_scratch_bytes(int K, int nsm);
