@@ -239,6 +239,7 @@ struct Layout {
   size_t at;         // column-major logA copy of the streamed configurations (256 < K <= 1024)
   size_t prune;      // bounded-row engine: copies and column lists of the largest model, then
   size_t guess, guess_bytes;  // the trace's segment ends
+  size_t give, give_wide;     // sequences handed to the other engines, the whole-GPU engine's scratch for them
   int32_t unit;               // table elements of a step at least
   uint64_t aux_elems;
   int64_t map_stride, snap_stride, list_cap;
@@ -305,7 +306,9 @@ Layout layout_for(const fv_model* models, int32_t n_models, const fv_batch* b, i
     L.unit = 128;
     for (int m = 0; m < n_models; ++m) L.unit = std::min(L.unit, models[m].K);
     L.guess_bytes = prune_guess_bytes(aux, n, sum_T, L.unit);
-    L.total = align_up(end + L.guess + L.guess_bytes);
+    L.give = align_up(L.guess + L.guess_bytes);
+    L.give_wide = align_up(L.give + sizeof(int32_t) * (kGiveStat + (size_t)n));
+    L.total = align_up(end + L.give_wide + (kmax > 1024 ? wide_state_bytes(kmax, device_sm_count()) : 0));
     return L;
   }
   if (beam0) {
@@ -476,6 +479,19 @@ size_t device_memory_bytes() {
     return (size_t)284208 << 20;  // no device visible: GB300's
   }
   return total;
+}
+
+// Whole-GPU engine scratch (wide_state_bytes) at w; returns its end.
+char* wide_state(DenseArgs* da, char* w) {
+  const size_t lanes_k = (size_t)kWideLanes * wide_lane_stride(da->K);
+  da->wide_D = reinterpret_cast<float*>(w);
+  w += align_up(2 * sizeof(float) * lanes_k);
+  da->wide_M = reinterpret_cast<uint16_t*>(w);
+  w += align_up(2 * sizeof(uint16_t) * lanes_k);
+  da->wide_X = reinterpret_cast<float*>(w);
+  w += align_up(2 * sizeof(float) * lanes_k);
+  da->wide_flags = reinterpret_cast<uint32_t*>(w);
+  return w + align_up(sizeof(uint32_t) * 8 * (size_t)(device_sm_count() + 1));
 }
 
 // Beam search (P = 0) and FLASH-BS (P >= 1) launch sequence, per model.
@@ -826,6 +842,7 @@ fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* ba
     if (prune) {
       da.kind = kJobVanilla;
       da.pr_D = reinterpret_cast<float*>(ws + L.aux);
+      da.give_stat = reinterpret_cast<int32_t*>(ws + L.prune + L.give);
       if (md.K > 128 && launch_prune_prep(md.logA, md.K, ws + L.prune, &da, st) != cudaSuccess) return FV_ECUDA;
       int64_t sum_T = 0, all_T = 0;
       int32_t max_T = 1;
@@ -835,6 +852,11 @@ fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* ba
         sum_T += batch->T_host[i];
         max_T = std::max(max_T, batch->T_host[i]);
       }
+      if (md.K > 128) {
+        prune_give(&da, md.K, R.count[m], max_T, !(p->flags & FV_SHARED_GPU));
+        da.give_list = da.give_stat + kGiveStat;
+        da.give_count = &hdr->given[m];
+      }
       timed_begin(st);
       if ((md.K <= 128 ? launch_small_values(da, st) : launch_prune_forward(da, sum_T, max_T, st)) != cudaSuccess)
         return FV_ECUDA;
@@ -842,6 +864,28 @@ fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* ba
       if (launch_prune_trace(da, reinterpret_cast<int32_t*>(ws + L.prune + L.guess), L.guess_bytes, all_T, L.unit, max_T,
                              paths_out, st) != cudaSuccess)
         return FV_ECUDA;
+      if (da.give_b > 0.f) {
+        // the sequences given up, with backpointer rows in the place of
+        // their (and of traced sequences') delta rows; none: three launches
+        // that end at once
+        da.order = da.give_list;
+        da.order_begin = 0;
+        da.order_live = da.give_count;
+        da.psi = reinterpret_cast<uint16_t*>(ws + L.aux);
+        int kpm = 0, cols = 0;
+        dense_stream_geometry(md.K, &kpm, &cols);
+        if (kpm) {
+          float2* pairs = reinterpret_cast<float2*>(ws + L.prune);
+          da.Ap = pairs;
+          da.ap_stride = cols;
+          if (launch_ap_prep(md.logA, md.K, pairs, st, da.order_live) != cudaSuccess) return FV_ECUDA;
+        }
+        if (md.K > 1024) wide_state(&da, ws + L.prune + L.give_wide);
+        if (launch_dense_forward(da, 0, st) != cudaSuccess) return FV_ECUDA;
+        if (launch_backtrack(jobs, da.order, 0, R.count[m], md.K, da.psi, qlast, paths_out, hdr, st, da.order_live) !=
+            cudaSuccess)
+          return FV_ECUDA;
+      }
       continue;
     }
     {
@@ -860,18 +904,7 @@ fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* ba
         }
       }
       if (md.K > 1024) {
-        // whole-GPU engine scratch: the same carving as wide_scratch_bytes
-        const size_t lanes_k = (size_t)kWideLanes * wide_lane_stride(md.K);
-        char* w = ws + L.wide;
-        da.wide_D = reinterpret_cast<float*>(w);
-        w += align_up(2 * sizeof(float) * lanes_k);
-        da.wide_M = reinterpret_cast<uint16_t*>(w);
-        w += align_up(2 * sizeof(uint16_t) * lanes_k);
-        da.wide_X = reinterpret_cast<float*>(w);
-        w += align_up(2 * sizeof(float) * lanes_k);
-        da.wide_flags = reinterpret_cast<uint32_t*>(w);
-        w += align_up(sizeof(uint32_t) * 8 * (size_t)(device_sm_count() + 1));
-        float* at = reinterpret_cast<float*>(w);
+        float* at = reinterpret_cast<float*>(wide_state(&da, ws + L.wide));
         da.wide_AT = at;
         if (launch_wide_transpose(md.logA, md.K, at, st) != cudaSuccess) return FV_ECUDA;
       }

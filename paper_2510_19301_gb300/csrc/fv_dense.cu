@@ -50,7 +50,10 @@ __global__ void __launch_bounds__(1024) prep_kernel(PrepArgs p) {
     p.hdr->detail = 0;
     carry = 0;
   }
-  for (int k = tid; k < kMaxModels; k += blockDim.x) p.hdr->pop[k] = 0ull;
+  for (int k = tid; k < kMaxModels; k += blockDim.x) {
+    p.hdr->pop[k] = 0ull;
+    p.hdr->given[k] = 0;
+  }
   if (tid < 5) p.hdr->counters[tid] = 0ull;
   __syncthreads();
   for (int base = 0; base < p.n_seq; base += blockDim.x) {
@@ -301,6 +304,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) dense_fwd_kernel(DenseArgs a) {
   __shared__ uint32_t s_info[2][5];  // per tick parity: active / MidState / sub-snapshot / drawn / ended slot masks
   __shared__ int s_abort;
 
+  if (a.order_live && *a.order_live <= 0) return;  // nothing was handed over (the same in every CTA)
   const int K = a.K;
   // resident: logA column slab as row pairs sA2[i/2][jj] = (A[i][j0+jj],
   // A[i+1][j0+jj]); streamed: each warp's ring of row-pair stages, filled
@@ -352,7 +356,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) dense_fwd_kernel(DenseArgs a) {
     const unsigned long long k = atomicAdd(a.pop, 1ull);
     const bool from_tasks = kind == kJobSub || kind == kJobLeaf;
     if (!from_tasks) {
-      if (k < (unsigned long long)a.order_count) {
+      if (k < (unsigned long long)(a.order_live ? *a.order_live : a.order_count)) {
         const int b = a.order[a.order_begin + (int)k];
         const Job jb = a.jobs[b];
         pj.valid = 1;
@@ -1194,11 +1198,12 @@ __global__ void __launch_bounds__(NW * 32, MINB) dense_fwd_kernel(DenseArgs a) {
 __global__ void __launch_bounds__(128) backtrack_kernel(const Job* jobs, const int32_t* order,
                                                         int32_t begin, int32_t count, int32_t K,
                                                         const uint16_t* psi, const int32_t* qlast,
-                                                        int32_t* paths, int32_t D, const WsHeader* hdr) {
+                                                        int32_t* paths, int32_t D, const WsHeader* hdr,
+                                                        const int32_t* live) {
   extern __shared__ __align__(16) uint16_t sbuf[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int idx = blockIdx.x * (blockDim.x >> 5) + warp;
-  if (idx >= count || hdr->status != 0) return;  // no forward pass ran: nothing to follow
+  if (idx >= (live ? *live : count) || hdr->status != 0) return;  // no forward pass ran: nothing to follow
   const int b = order[begin + idx];
   const Job jb = jobs[b];
   uint16_t* buf = sbuf + (size_t)warp * D * K;
@@ -1403,7 +1408,8 @@ void dense_stream_geometry(int K, int* KPM, int* cols) {
   *cols = 1024;
 }
 
-__global__ void ap_prep_kernel(const float* logA, int K, int KPM, int cols, float2* Ap) {
+__global__ void ap_prep_kernel(const float* logA, int K, int KPM, int cols, float2* Ap, const int32_t* live) {
+  if (live && *live <= 0) return;
   const int64_t n = (int64_t)(KPM / 2) * cols;
   for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
     const int ip = (int)(x / cols), c = (int)(x % cols), i = 2 * ip;
@@ -1413,11 +1419,11 @@ __global__ void ap_prep_kernel(const float* logA, int K, int KPM, int cols, floa
   }
 }
 
-cudaError_t launch_ap_prep(const float* logA, int K, float2* Ap, cudaStream_t st) {
+cudaError_t launch_ap_prep(const float* logA, int K, float2* Ap, cudaStream_t st, const int32_t* live) {
   int KPM, cols;
   dense_stream_geometry(K, &KPM, &cols);
   if (!KPM) return cudaSuccess;
-  ap_prep_kernel<<<1024, 256, 0, st>>>(logA, K, KPM, cols, Ap);
+  ap_prep_kernel<<<live ? 2 * device_sm_count() : 1024, 256, 0, st>>>(logA, K, KPM, cols, Ap, live);
   return cudaGetLastError();
 }
 
@@ -1539,7 +1545,7 @@ cudaError_t launch_order(const Job* jobs, int32_t n, int32_t nosort, int32_t* or
 
 cudaError_t launch_backtrack(const Job* jobs, const int32_t* order, int32_t begin, int32_t count,
                              int32_t K, const uint16_t* psi, const int32_t* qlast, int32_t* paths,
-                             const WsHeader* hdr, cudaStream_t st) {
+                             const WsHeader* hdr, cudaStream_t st, const int32_t* live) {
   if (count <= 0) return cudaSuccess;
   int D = 16384 / (2 * K);
   if (D < 1) D = 1;
@@ -1549,7 +1555,7 @@ cudaError_t launch_backtrack(const Job* jobs, const int32_t* order, int32_t begi
   cudaError_t e = cudaFuncSetAttribute(backtrack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   backtrack_kernel<<<(count + warps - 1) / warps, warps * 32, smem, st>>>(jobs, order, begin, count, K, psi,
-                                                                       qlast, paths, D, hdr);
+                                                                       qlast, paths, D, hdr, live);
   return cudaGetLastError();
 }
 

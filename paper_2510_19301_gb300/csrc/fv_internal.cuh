@@ -30,7 +30,8 @@ struct WsHeader {
   uint64_t aux_cap;            // elements available
   uint64_t counters[5];        // mode-specific counters (tasks, reruns, ...)
   unsigned long long pop[kMaxModels];  // per-model work counters
-  uint32_t pad[(1024 - 64 - 8 * kMaxModels) / 4];
+  int32_t given[kMaxModels];  // per model: sequences the bounded-row engine handed back
+  uint32_t pad[(1024 - 64 - 12 * kMaxModels) / 4];
 };
 static_assert(sizeof(WsHeader) == 1024, "header must be 1 KiB");
 
@@ -121,6 +122,13 @@ __device__ inline void st_async_v4(uint32_t addr, uint4 v, uint32_t remote_bar) 
   asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
                    addr),
                "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(remote_bar)
+               : "memory");
+}
+
+// the same with one word
+__device__ inline void st_async_u32(uint32_t addr, uint32_t v, uint32_t remote_bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(v),
+               "r"(remote_bar)
                : "memory");
 }
 

@@ -143,6 +143,16 @@ struct DenseArgs {
   int32_t beam_stride;
   int32_t* beam_id;
   float* beam_val;
+  // sequences handed from the bounded-row engine to the others: time of a
+  // step with r rows, a + b r, in units of the other engine's step (b = 0:
+  // none is), the launch's row counts (kGiveStat words, cleared by the
+  // preparation), the list of them and its length; order_live: the other
+  // engine's number of sequences, read there
+  float give_a, give_b;
+  int32_t* give_stat;
+  int32_t* give_list;
+  int32_t* give_count;
+  const int32_t* order_live;
   int32_t no_tune;            // use the default engine configuration, not the tuned one
   WsHeader* hdr;
 };
@@ -234,7 +244,8 @@ void dense_set_variant(int K, bool table, int v);
 int dense_get_variant(int K, bool table);
 int device_sm_count();
 bool wide_geometry(int K, int nsm, WideGeom* g);
-size_t wide_scratch_bytes(int K, int nsm);
+size_t wide_state_bytes(int K, int nsm);    // what the engine keeps between steps
+size_t wide_scratch_bytes(int K, int nsm);  // that and the column-major copy of logA
 cudaError_t launch_wide_forward(DenseArgs a, cudaStream_t st);
 // small state spaces (K <= 128), every job kind: a CTA of K-class threads per
 // job, a thread per state (fv_small.cu)
@@ -245,6 +256,10 @@ cudaError_t launch_small_forward(const DenseArgs& a, cudaStream_t st);
 size_t prune_area_bytes(int K);
 cudaError_t launch_prune_prep(const float* logA, int K, char* area, DenseArgs* a, cudaStream_t st);
 cudaError_t launch_prune_forward(const DenseArgs& a, int64_t sum_T, int max_T, cudaStream_t st);
+constexpr int kGiveStat = 64;
+// when a sequence of this launch is better handed to the other engines
+// (sets give_a and give_b)
+void prune_give(DenseArgs* a, int K, int jobs, int max_T, bool alone);
 size_t prune_guess_bytes(uint64_t aux_elems, int32_t n_seq, int64_t sum_T, int32_t unit);
 cudaError_t launch_prune_trace(const DenseArgs& a, int32_t* guess, size_t guess_bytes, int64_t sum_T, int unit,
                                int max_T, int32_t* paths, cudaStream_t st);
@@ -261,13 +276,15 @@ cudaError_t launch_small_values(const DenseArgs& a, cudaStream_t st);
 // AT[j * KD + i] = logA[i * K + j] (rows K..KD-1 are -inf), KD = wide_lane_stride(K).
 cudaError_t launch_wide_transpose(const float* logA, int K, float* AT, cudaStream_t st);
 void dense_stream_geometry(int K, int* KPM, int* cols);
-cudaError_t launch_ap_prep(const float* logA, int K, float2* Ap, cudaStream_t st);
+// live (may be null): the number of sequences, on the device, without any of
+// which the launch does nothing
+cudaError_t launch_ap_prep(const float* logA, int K, float2* Ap, cudaStream_t st, const int32_t* live = nullptr);
 cudaError_t launch_prep(const PrepArgs& p, cudaStream_t st);
 cudaError_t launch_order(const Job* jobs, int32_t n, int32_t nosort, int32_t* order, cudaStream_t st);
 cudaError_t launch_dense_forward(DenseArgs a, int max_clusters, cudaStream_t st);
 cudaError_t launch_backtrack(const Job* jobs, const int32_t* order, int32_t begin, int32_t count, int32_t K,
                              const uint16_t* psi, const int32_t* qlast, int32_t* paths, const WsHeader* hdr,
-                             cudaStream_t st);
+                             cudaStream_t st, const int32_t* live = nullptr);
 cudaError_t launch_flash_resolve(const Job* jobs, const int32_t* order, int32_t begin, int32_t count,
                                  int32_t K, int32_t P, const uint16_t* maps, const float* snaps,
                                  int64_t map_stride, int64_t snap_stride, int32_t* paths, float* sval,

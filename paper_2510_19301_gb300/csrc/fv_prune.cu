@@ -17,7 +17,8 @@
 // Only the maximum is kept: delta_t = fl(max + E_t) is exact on any input (an
 // input that bounds badly only runs more rows), delta rows go to the
 // workspace, and the backtrack recomputes the argmax of the path's own states
-// (below), K candidates per step instead of K^2 backpointers.  On Dirichlet(1)
+// (below), K candidates per step instead of K^2 backpointers.  A sequence that
+// forms too many rows is handed to the other engines (prune_give).  On Dirichlet(1)
 // weights with log-softmax normal emissions a step takes about 34 of 256 rows,
 // 40 of 512, 61 of 1000.
 //
@@ -38,6 +39,8 @@
 
 namespace fv {
 
+constexpr int kGiveLevels = 31;  // votes on handing a sequence over (below)
+
 // ------------------------------------------------------------------- prep
 // Order-preserving key of a float (larger float, larger key); 0 is below
 // every key of a number.
@@ -57,10 +60,12 @@ __device__ __forceinline__ float ord_value(uint32_t k) {
 // that global loads read whole 32-byte sectors.
 template <int VPL>
 __global__ void __launch_bounds__(256) prune_prep_kernel(const float* logA, int K, int KP, int M, float* Apad,
-                                                         float* AT, float* lval, uint16_t* lrow, float* cut) {
+                                                         float* AT, float* lval, uint16_t* lrow, float* cut,
+                                                         int32_t* stat) {
   extern __shared__ float scol[];  // [8][32 * VPL + 4]
   constexpr int ST = 32 * VPL + 4;
   const int j0 = blockIdx.x * 8, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (stat && blockIdx.x == 0 && tid < 2 * kGiveLevels) stat[tid] = 0;
   for (int x = tid; x < 8 * K; x += 256) {
     const int i = x >> 3, c = x & 7;
     const float v = j0 + c < K ? __ldg(logA + (int64_t)i * K + j0 + c) : -CUDART_INF_F;
@@ -219,15 +224,62 @@ struct PruneCfg {
 // bounded wait of the cluster exchange (~1 s at 2 GHz)
 constexpr long long kPruneWaitCycles = 1ll << 31;
 
+// Before steps t = 8, 16, 32, ... a job's warps, in all of its CTAs, tell each
+// other how many rows per step they have formed since the last time (the most
+// of any warp sets the step's time), and agree whether the sequence is handed
+// over.  The launch's jobs add theirs up, and a sequence leaves where the steps
+// left to it, at a + b rows each, take longer than all its steps there (unit:
+// a step there) by the average of the time before, so that like sequences
+// leave together and the other engine is not run beside half a launch; or
+// where by its own rows they take kGiveAlone times as long.
+constexpr float kGiveAlone = 2.5f;
+__device__ __forceinline__ bool give_longer(float rows, float times, float ga, float gb, int t, int T) {
+  return (float)(T - t) * __fmaf_rn(gb, rows, ga) > times * (float)T;
+}
+// A warp's word: its rows, and in the high half whether the launch's average
+// says to leave.  (Not inlined: its registers are not the step loop's.)
+__device__ __noinline__ uint32_t give_word(const int32_t* stat, uint32_t rows, float ga, float gb, int t, int T) {
+  const volatile int32_t* s = stat + 2 * (30 - __clz(t));
+  const int sum = s[0], n = s[1];
+  const bool leave = n > 0 && give_longer((float)sum / (float)n, 1.f, ga, gb, t, T);
+  return (rows < 0xffffu ? rows : 0xffffu) | (leave ? 0x10000u : 0u);
+}
+// The job's decision, from all words; `lead`: one thread of the job.
+__device__ __forceinline__ bool give_decide(const uint32_t* words, int n, int32_t* stat, bool lead, float ga, float gb,
+                                         int t, int T) {
+  uint32_t most = 0, leave = 0;
+#pragma unroll 1
+  for (int x = 0; x < n; ++x) {
+    const uint32_t w = words[x];
+    most = max(most, w & 0xffffu);
+    leave |= w >> 16;
+  }
+  if (lead) {
+    int32_t* s = stat + 2 * (31 - __clz(t));
+    atomicAdd(s, (int)most);
+    atomicAdd(s + 1, 1);
+  }
+  return leave != 0 || give_longer((float)most, kGiveAlone, ga, gb, t, T);
+}
+
 template <int KP, int CL, int C, int G, bool RES, int M, bool BEAM>
 __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M, BEAM>::NT, 1) prune_fwd_kernel(DenseArgs a) {
   using Cfg = PruneCfg<KP, CL, C, G, RES, M, BEAM>;
   constexpr int KH = Cfg::KH, W = Cfg::W, NT = Cfg::NT, NW = Cfg::NW, CAP = Cfg::CAP, WB = Cfg::WB, U = Cfg::U;
   constexpr bool COOP = Cfg::COOP;
+  constexpr bool GIVE = !BEAM && KP > 256;  // sequences may be handed to the other engines
+  // where the votes on that are taken: between runs of the step loop, or at
+  // its top (by what the compiler makes of the loop: one K = 512 sequence 1.38
+  // / 1.42 ms, 150 K = 1000 sequences 7.55 / 7.05, 8 K = 4096 ones 21.0 / 17.8)
+  constexpr bool LOOK_OUT = GIVE && KP == 512;
   extern __shared__ __align__(16) char smem[];
   __shared__ __align__(8) uint64_t s_bar[G][2];
   __shared__ int s_abort;
   __shared__ uint32_t s_stop[CL];
+  __shared__ __align__(8) uint64_t s_wbar[G];     // the words of a job's other CTAs are here
+  __shared__ uint32_t s_votes[GIVE ? G : 1][W];     // exchanges of words so far, per warp
+  __shared__ int s_rows[GIVE ? G : 1][W];           // rows formed since the last one, per warp
+  __shared__ uint32_t s_word[GIVE ? G : 1][CL][W];  // what the warps say (give_word)
   __shared__ float s_max[G][W], s_need[G][2][W];  // COOP: per warp maxima and depths
   __shared__ int s_cnt[G][2][2];                  // COOP: entries of the common lists, by step parity
   // BEAM: candidates per bin (by step parity), those of the bin that holds
@@ -290,6 +342,7 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M, BEAM>::NT, 1) p
   uint32_t peer[2] = {0u, 0u};  // CL = 2: shared memory of either CTA
   const uint32_t self = smem_addr(smem);
   if (threadIdx.x == 0) s_abort = 0;
+  if (GIVE && lane == 0) s_votes[grp][gw] = 0;
   if constexpr (CL > 1) {
     if constexpr (CL == 2) {
       peer[0] = dsmem_addr(smem, 0);
@@ -297,6 +350,7 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M, BEAM>::NT, 1) p
     }
     if (threadIdx.x < 2 * G) {
       mbar_init(smem_addr(&s_bar[0][0] + threadIdx.x), 1);
+      if (threadIdx.x < G) mbar_init(smem_addr(&s_wbar[threadIdx.x]), 1);
       fence_mbar_init_cluster();
     }
     cluster_sync_all();  // every CTA of the cluster runs and its barriers are ready
@@ -317,7 +371,7 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M, BEAM>::NT, 1) p
   const int ncl = (int)gridDim.x / CL, slots = ncl * G;
   const int cid = (int)blockIdx.x / CL;
   const int slot = grp * ncl + ((grp & 1) ? ncl - 1 - cid : cid);
-  bool live = true, dead = false;
+  bool live = true, dead = false, gave = false;
   uint32_t ph = 0;  // steps run so far: buffer ph & 1, its (ph >> 1)-th use
 
   for (int round = 0;; ++round) {
@@ -368,7 +422,47 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M, BEAM>::NT, 1) p
       // (ordered by the barriers of the first step)
     }
     float gap = 0.f;  // how far below the maximum this warp's last steps had to look
-    for (int t = 0; t < T; ++t, ++ph) {
+    // hand the sequence over before step t?  (or, `live` false, a wait ran out)
+    auto stop_before = [&](int t) -> bool {
+      constexpr int g0 = GIVE ? 1 : 0;
+      const uint32_t rows = (uint32_t)s_rows[g0 * grp][gw] / (uint32_t)(t == 8 ? 8 : t / 2);
+      __syncwarp();
+      if (lane == 0) s_rows[g0 * grp][gw] = 0;
+      const uint32_t word = give_word(a.give_stat, rows, a.give_a, a.give_b, t, T);
+      if (lane == 0) s_word[g0 * grp][rank][gw] = word;
+      bool late = false;
+      if constexpr (CL > 1) {
+        const uint32_t bar = smem_addr(&s_wbar[grp]), par = s_votes[g0 * grp][gw] & 1u;
+        if (gt == 0) mbar_arrive_expect_tx(bar, (CL - 1) * W * 4);
+        if (lane < CL && lane != (int)rank)
+          st_async_u32(dsmem_addr(&s_word[g0 * grp][rank][gw], lane), word, dsmem_addr(&s_wbar[grp], lane));
+        const long long w0 = clock64();
+        while (!late && !mbar_try_wait_cluster(bar, par))
+          late = *(volatile int*)&s_abort || clock64() - w0 > kPruneWaitCycles;
+      }
+      __syncwarp();
+      if (lane == 0) ++s_votes[g0 * grp][gw];
+      if (group_any(late)) {
+        // (as at the end of a step, below)
+        set_status(a.hdr, FV_ETIMEOUT, 6);
+        *(volatile int*)&s_abort = 1;
+        const long long w0 = clock64();
+        while (clock64() - w0 < (1ll << 18)) {
+        }
+        live = false;
+        return true;
+      }
+      gave = give_decide(&s_word[g0 * grp][0][0], CL * W, a.give_stat, rank == 0 && gt == 0, a.give_a, a.give_b, t, T);
+      return gave;
+    };
+    if (GIVE && lane == 0) s_rows[grp][gw] = 0;
+    int t = 0, look = LOOK_OUT && a.give_b > 0.f && T > 8 ? 8 : T;
+  steps:
+    __attribute__((unused));
+    for (; t < (LOOK_OUT ? look : T); ++t, ++ph) {
+      if constexpr (GIVE && !LOOK_OUT) {
+        if (t >= 8 && (t & (t - 1)) == 0 && a.give_b > 0.f && stop_before(t)) break;
+      }
       const uint32_t cur = ph & 1u;  // buffer written by this step; cur ^ 1 is read
       float e[C];
 #pragma unroll
@@ -683,6 +777,7 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M, BEAM>::NT, 1) p
         };
         // the listed rows (their order does not matter: only the maximum is kept)
         auto flush = [&](int n) {
+          if (GIVE && lane == 0) s_rows[grp][gw] += n;
           close_list(list, n);
 #pragma unroll 1
           for (int i = 0; i < n; i += U) {
@@ -720,6 +815,7 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M, BEAM>::NT, 1) p
             }
           }
         }
+        if (GIVE && lane == 0) s_rows[grp][gw] += n;
         close_list(first, n);  // (every warp writes the same beyond a common list)
         load_rows(first, 0);
 #pragma unroll
@@ -889,7 +985,21 @@ __global__ void __launch_bounds__(PruneCfg<KP, CL, C, G, RES, M, BEAM>::NT, 1) p
         break;
       }
     }
+    if constexpr (LOOK_OUT) {
+      if (live && t < T && !stop_before(t)) {
+        look = 2 * look < T ? 2 * look : T;
+        goto steps;
+      }
+    }
     if (!live) break;
+    if (GIVE && gave) {
+      gave = false;
+      if (rank == 0 && gt == 0) {
+        a.qlast[b] = -1;  // nothing to trace
+        a.give_list[atomicAdd(a.give_count, 1)] = b;
+      }
+      continue;
+    }
     if (BEAM && dead) {
       // the same in every CTA of the cluster, before anything of the step was
       // exchanged; the next job clears what this one read
@@ -1102,6 +1212,7 @@ __global__ void __launch_bounds__(32 * TW) prune_trace_kernel(TraceArgs a) {
   const int b = a.order[a.begin + blockIdx.x];
   const Job jb = a.jobs[b];
   const int T = jb.T, K = a.K;
+  if (a.qlast[b] < 0) return;  // handed to another engine
   Tracer<VPL, TW, BEAM, ROWS> tr;
   tr.init(a, jb, part);
   int32_t* path = a.paths + jb.path_off;
@@ -1139,6 +1250,7 @@ __global__ void __launch_bounds__(32 * TW) prune_fix_kernel(TraceArgs a) {
   if (a.hdr->status != 0) return;
   const int b = a.order[a.begin + blockIdx.x], lane = threadIdx.x & 31;
   const Job jb = a.jobs[b];
+  if (a.qlast[b] < 0) return;
   const int K = a.K, nseg = (jb.T + a.seg - 1) / a.seg;
   int32_t* path = a.paths + jb.path_off;
   const int64_t g0 = guess_off(a, jb, b);
@@ -1181,29 +1293,37 @@ int prune_pad(int K) { return K <= 256 ? 256 : K <= 512 ? 512 : K <= 1024 ? 1024
 // 2.18 / 2.07; K = 1000, 8 / 12 / 16: 152 sequences 9.1 / 8.9 / 8.6.  A longer
 // list lowers the cutoffs (fewer rows) but gathers more deltas.
 int prune_list(int K) { return K <= 256 ? 6 : K <= 512 ? 12 : K <= 1024 ? 16 : 32; }
+// the row copy, and in its place the row-pair copy of the engine that
+// sequences are handed to once the others are traced
+static size_t prune_copy_bytes(int K) {
+  int kpm = 0, cols = 0;
+  dense_stream_geometry(K, &kpm, &cols);
+  const size_t rows = (size_t)K * prune_pad(K) * 4, pairs = (size_t)kpm * cols * 4;
+  return align_up(rows > pairs ? rows : pairs);
+}
 // area: row copy, column-major copy, list values, cutoffs, list rows
 size_t prune_area_bytes(int K) {
   if (K <= 128) return 0;  // (fv_small.cu needs none)
   const size_t KP = prune_pad(K), M = prune_list(K);
-  return align_up((size_t)K * KP * 4) + align_up((size_t)K * wide_lane_stride(K) * 4) + align_up(KP * (M * 6 + 4));
+  return prune_copy_bytes(K) + align_up((size_t)K * wide_lane_stride(K) * 4) + align_up(KP * (M * 6 + 4));
 }
 
 template <int VPL>
 static cudaError_t launch_prep_cfg(const float* logA, int K, float* A, float* at, float* val, uint16_t* row, float* cut,
-                                   cudaStream_t st) {
+                                   int32_t* stat, cudaStream_t st) {
   const size_t sm = 8 * (32 * VPL + 4) * sizeof(float);
   cudaError_t e =
       cudaFuncSetAttribute(prune_prep_kernel<VPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   prune_prep_kernel<VPL><<<prune_pad(K) / 8, 256, sm, st>>>(logA, K, prune_pad(K), prune_list(K), A, at, val, row,
-                                                              cut);
+                                                              cut, stat);
   return cudaGetLastError();
 }
 
 cudaError_t launch_prune_prep(const float* logA, int K, char* area, DenseArgs* a, cudaStream_t st) {
   const int KP = prune_pad(K), M = prune_list(K);
   float* copy = reinterpret_cast<float*>(area);
-  area += align_up((size_t)K * KP * 4);
+  area += prune_copy_bytes(K);
   float* at = reinterpret_cast<float*>(area);
   area += align_up((size_t)K * wide_lane_stride(K) * 4);
   float* val = reinterpret_cast<float*>(area);
@@ -1214,11 +1334,11 @@ cudaError_t launch_prune_prep(const float* logA, int K, char* area, DenseArgs* a
   a->pr_row = row;
   a->pr_cut = cut;
   a->wide_AT = at;
-  if (K <= 256) return launch_prep_cfg<8>(logA, K, copy, at, val, row, cut, st);
-  if (K <= 512) return launch_prep_cfg<16>(logA, K, copy, at, val, row, cut, st);
-  if (K <= 1024) return launch_prep_cfg<32>(logA, K, copy, at, val, row, cut, st);
-  if (K <= 2048) return launch_prep_cfg<64>(logA, K, copy, at, val, row, cut, st);
-  return launch_prep_cfg<128>(logA, K, copy, at, val, row, cut, st);
+  if (K <= 256) return launch_prep_cfg<8>(logA, K, copy, at, val, row, cut, a->give_stat, st);
+  if (K <= 512) return launch_prep_cfg<16>(logA, K, copy, at, val, row, cut, a->give_stat, st);
+  if (K <= 1024) return launch_prep_cfg<32>(logA, K, copy, at, val, row, cut, a->give_stat, st);
+  if (K <= 2048) return launch_prep_cfg<64>(logA, K, copy, at, val, row, cut, a->give_stat, st);
+  return launch_prep_cfg<128>(logA, K, copy, at, val, row, cut, a->give_stat, st);
 }
 
 // Clusters (CTAs for CL = 1) of a configuration resident at once; 0 where the
@@ -1314,6 +1434,56 @@ cudaError_t launch_prune_forward(const DenseArgs& a, int64_t sum_T, int max_T, c
   }
   if (a.K <= 2048) return launch_prune_cfg<2048, 4, 2, 1, false, 32, false>(a, st);
   return launch_prune_cfg<4096, 8, 2, 1, false, 32, false>(a, st);
+}
+
+// When a sequence is handed to the other engines.  Inputs whose bounds prune
+// little (smooth position models, blocks of states, ties) make it read nearly
+// every row for itself, where those engines share a row among the sequences
+// of a cluster or of the GPU.  Measured (GB300, us per step of the launch):
+//                  ordinary  ties  Gaussian band  all equal   other engine
+//   K = 512,    64    2.8     4.1       7.3          8.1          4.1
+//              152    3.0     5.0       9.2         11.3          7.7
+//              400    8.0    14.6      28.3         35.4         15.2
+//   K = 1000,   60    4.6    10.9      21.6         27.9         11.2
+//              152    6.4    14.9      28.4         37.7         26.6
+//   K = 1500,    4    4.7    11.9      20.0         30.0         11.2
+//   K = 2048,    8    5.8    15.9      27.2         40.4         13.2
+//   K = 4096,    8   11.8    37.3      55.0        100.6         20.1
+// With the rule, us per step: K = 4096, 8 sequences of 600 steps, band 54 -> 22.6,
+// all equal 99 -> 21.3 (the other engine alone 19.7); K = 1000, one of 1500,
+// 18.4 -> 11.7 and 26.4 -> 10.8 (10.6); K = 512, 64 of 200, all equal 8.1 -> 4.8
+// (4.1); 100 steps at K = 4096, all equal 91 -> 29: the shorter a sequence, the
+// more of it is gone before the rule can tell.
+// The constants are a line a + b rows through these (rows of the busiest
+// warp) and the other engine's step; sequences have to lose 15%.  Where none
+// is handed over the call pays launches that end at once (9 to 13 us), so it
+// does without where that is more than a few percent of it: short calls, K
+// <= 256 (all equal 16.9 against 13.6) and the few states where reading every
+// row loses less than 30%.  Above K = 1024 the other engine waits for the whole
+// GPU, so calls that share it do without too.
+void prune_give(DenseArgs* a, int K, int jobs, int max_T, bool alone) {
+  const int nsm = device_sm_count();
+  a->give_a = a->give_b = 0.f;
+  if (K <= 256 || max_T < (K <= 512 ? 128 : K <= 2048 ? 64 : 32) || (K > 1024 && !alone)) return;
+  float ca, cb, there;
+  if (K <= 512) {
+    if (jobs <= 120) ca = 1.7f, cb = 0.0125f, there = 4.05f;
+    else if (jobs <= nsm) ca = 1.7f, cb = 0.0185f, there = 7.7f;
+    else ca = 1.2f, cb = 0.0225f, there = 5.8f;  // per 152 sequences
+  } else if (K <= 1024) {
+    if (2 * jobs <= nsm) ca = 1.5f, cb = 0.023f, there = 11.f;
+    else ca = 2.5f, cb = 0.034f, there = 11.f + 15.6f * fminf(1.f, 2.f * (float)jobs / (float)nsm - 1.f);
+  } else {
+    // kWideLanes sequences at a time there, a cluster each here
+    const int resident = K <= 2048 ? nsm / 4 - 2 : nsm / 8 - 4;
+    const float turns = (float)((jobs + resident - 1) / resident);
+    ca = (K <= 2048 ? 3.2f : 5.f) * turns;
+    cb = (K <= 2048 ? 0.0175f : 5.25e-6f * (float)K) * turns;
+    there = (5.5f + 0.0036f * (float)K) * (float)((jobs + kWideLanes - 1) / kWideLanes);
+  }
+  if (ca + cb * (float)K < 1.3f * there) return;
+  a->give_a = ca / (1.15f * there);
+  a->give_b = cb / (1.15f * there);
 }
 
 // States per segment of the trace: a few thousand segments over the launch,

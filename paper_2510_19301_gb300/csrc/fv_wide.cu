@@ -189,13 +189,15 @@ bool wide_geometry(int K, int nsm, WideGeom* g) {
   return true;
 }
 
-size_t wide_scratch_bytes(int K, int nsm) {
-  // delta and MidState double buffers, sub snapshots (job parity), flags,
-  // and the column-major copy of logA read by the owners' re-scan
+size_t wide_state_bytes(int K, int nsm) {
+  // delta and MidState double buffers, sub snapshots (job parity), flags
   const size_t lk = (size_t)kWS * wide_lane_stride(K);
   return align_up(2 * sizeof(float) * lk) + align_up(2 * sizeof(uint16_t) * lk) + align_up(2 * sizeof(float) * lk) +
-         align_up(sizeof(uint32_t) * 8 * (size_t)(nsm + 1)) +
-         align_up(sizeof(float) * (size_t)K * wide_lane_stride(K));
+         align_up(sizeof(uint32_t) * 8 * (size_t)(nsm + 1));
+}
+size_t wide_scratch_bytes(int K, int nsm) {
+  // and the column-major copy of logA read by the owners' re-scan
+  return wide_state_bytes(K, nsm) + align_up(sizeof(float) * (size_t)K * wide_lane_stride(K));
 }
 
 // 32 x 32 tiles through shared memory, so both sides are coalesced.
@@ -237,6 +239,7 @@ __global__ void __launch_bounds__(kWNT, 1) wide_fwd_kernel(DenseArgs a, WideGeom
     return;
   }
 
+  if (a.order_live && *a.order_live <= 0) return;  // nothing was handed over (the same in every CTA)
   const int K = a.K, RPC = g.RPC, RPW = g.RPW, RWR = g.RWR, RPCS = RPC + RPC / 8;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = cluster_ctarank();
@@ -268,7 +271,7 @@ __global__ void __launch_bounds__(kWNT, 1) wide_fwd_kernel(DenseArgs a, WideGeom
   }
   const bool from_tasks = kind == kJobSub || kind == kJobLeaf;
   const int task0 = from_tasks && a.task_first ? *a.task_first : 0;
-  if (tid == 0) s_njobs = from_tasks ? *a.task_count : a.order_count;
+  if (tid == 0) s_njobs = from_tasks ? *a.task_count : (a.order_live ? *a.order_live : a.order_count);
   if (tid < 2 * CR) s_abort[tid / CR][tid % CR] = 0;
   // producers of this CTA's rows: every CTA of the clusters covering them
   const int rows_hi = row0 + RPC < K ? row0 + RPC : K;
