@@ -1554,8 +1554,14 @@ cudaError_t launch_prune_trace(const DenseArgs& a, int32_t* guess, size_t guess_
 // B = 256, one sequence 12.0 -> 10.2, 64 sequences 34.7 -> 21.8), so the launch
 // is compared with one CTA per sequence on fv_beam.cu, whose step takes 3
 // times as long or more; K = 4096 was no faster (one sequence 17.8 -> 21.5).
-// Returns false where fv_beam.cu wins.
+// Short calls stay there too, where the preparation of logA outweighs the
+// steps: below 32 steps (48 from K = 1024) where fv_beam.cu would spread a
+// sequence over a cluster (one sequence of 3 / 20 / 200 steps: K = 1024, B = 256,
+// 51 / 185 / 1732 us there, 64 / 210 / 1390 here; K = 2048, B = 512, 72 / 302 / 2955
+// against 103 / 362 / 1902), else below 8 (K = 1000, B = 16, 48 / 226 / 2135
+// against 51 / 125 / 719).  Returns false where fv_beam.cu wins.
 bool prune_beam_wins(int K, int64_t sum_T, int max_T, bool alone) {
+  if (K >= 512 && max_T < (alone && K % 32 == 0 ? (K < 1024 ? 32 : 48) : 8)) return false;
   if (K <= 1024) return true;
   if (!alone || K > 2048) return false;
   const int64_t nsm = device_sm_count(), ncl = nsm / 4 - 2;
