@@ -757,12 +757,13 @@ fv_status fv_decode(const fv_model* models, int32_t n_models, const fv_batch* ba
     prune = p->mode == FV_BEAM ||
             dense_uses_prune(models[m].K, (p->flags & FV_NO_TUNE) != 0);
   // (preparing a model above K = 2048 costs more than the whole-GPU engine's
-  // steps up to about 30: K = 4096, 5 / 20 steps 326 / 497 against 210 / 482 us)
+  // steps up to about 30: K = 4096, 5 / 20 steps 326 / 497 against 210 / 482 us;
+  // for K <= 128 see small_values_win)
   if (prune && p->mode == FV_VANILLA) {
     int32_t kmax = 0, tmax = 0;
     for (int m = 0; m < n_models; ++m) kmax = std::max(kmax, models[m].K);
     for (int i = 0; i < n; ++i) tmax = std::max(tmax, batch->T_host[i]);
-    prune = kmax <= 2048 || tmax >= 32;
+    prune = kmax <= 128 ? small_values_win(kmax, n, tmax) : kmax <= 2048 || tmax >= 32;
   }
   if (prune) {
     const Layout LP = layout_for(models, n_models, batch, p->mode, nullptr, p->B, 0, true);

@@ -273,6 +273,8 @@ bool dense_prune_K(int K);
 bool dense_uses_prune(int K, bool no_tune);
 // exact decoding at K <= 128, values only: delta rows to a.pr_D (fv_small.cu)
 cudaError_t launch_small_values(const DenseArgs& a, cudaStream_t st);
+// whether that is faster than the kernel with backpointer rows
+bool small_values_win(int K, int jobs, int max_T);
 // AT[j * KD + i] = logA[i * K + j] (rows K..KD-1 are -inf), KD = wide_lane_stride(K).
 cudaError_t launch_wide_transpose(const float* logA, int K, float* AT, cudaStream_t st);
 void dense_stream_geometry(int K, int* KPM, int* cols);

@@ -511,6 +511,21 @@ __global__ void __launch_bounds__(KM + 32) small_value_kernel(DenseArgs a) {
   }
 }
 
+// A call of few steps is faster with backpointers: the start of this kernel
+// and the trace (a column of logA per step, where a backpointer is one
+// load) cost more than its steps save.  Measured, us per call, values /
+// backpointers: K = 64, one sequence of 64 / 128 / 256 steps 50 / 42, 68 / 66, 103 /
+// 114; K = 128 75 / 60, 105 / 105, 165 / 193; K = 16 44 / 41, 62 / 64, 94 / 109.
+// Where rows of K uint16 do not come in whole 16-byte pieces the backtrack is
+// slower and the line lower: K = 37, 24 / 48 / 96 steps 30 / 30, 39 / 40, 58 / 64; K
+// = 100 42 / 40, 58 / 58, 87 / 101.  So it is where the launch fills the GPU: K =
+// 128, 300 sequences of 24 / 48 steps 49 / 46, 66 / 72.
+bool small_values_win(int K, int jobs, int max_T) {
+  const bool many = jobs > (K > 64 ? 1 : 2) * device_sm_count();
+  if (K % 8 != 0 || many) return max_T >= 40;
+  return max_T >= (K > 32 && K <= 64 ? 144 : 112);
+}
+
 cudaError_t launch_small_values(const DenseArgs& a, cudaStream_t st) {
   if (a.K > 128) return cudaErrorInvalidValue;
   if (a.order_count <= 0) return cudaSuccess;
