@@ -169,9 +169,10 @@ typedef struct {
  * transitions only (FV_EUNSUPPORTED for CSR), K <= 4096.
  *
  * Supported: FV_VANILLA and FV_FLASH on dense transitions need
- * K <= 4096 (FV_EUNSUPPORTED otherwise); K > 1024 runs one cooperative
- * launch over the whole GPU whose device waits are bounded (FV_ETIMEOUT in
- * the status word if one runs out).  FV_BEAM takes dense or CSR
+ * K <= 4096 (FV_EUNSUPPORTED otherwise).  Waits between CTAs (clusters, and
+ * at K > 1024 one cooperative launch over the whole GPU where backpointers or
+ * MidState are kept) are bounded (FV_ETIMEOUT in the status word if one runs
+ * out).  FV_BEAM takes dense or CSR
  * transitions with K <= 65536.  A batch with a CSR model is decoded
  * exactly by the beam of Sec. V-C with every state kept (B = K; FLASH
  * becomes FLASH-BS with the same P), which gives the same paths and scores
@@ -250,8 +251,10 @@ fv_status fv_timing_read(float* total_ms, int32_t* n_pairs);
 /* The recorded pairs one by one (milliseconds each, in recording order, at
  * most max_pairs; *n_pairs = how many were written).  A FLASH decode records
  * one pair for its root pass (with the resolve) and one per task level of
- * Alg. 1 (the budget-leaf waves of the leaf level together); the other
- * modes one pair per decode.  Synchronises on the recorded pairs. */
+ * Alg. 1 run (the budget-leaf waves of the leaf level together; at K <= 128
+ * the first level that is solved directly is the last); the other modes one
+ * pair per model, without the trace and what exact decoding hands to another
+ * engine.  Synchronises on the recorded pairs. */
 fv_status fv_timing_pairs(float* ms, int32_t max_pairs, int32_t* n_pairs);
 
 /* Autotuning of the exact forward engine (not in the paper).  Dense exact

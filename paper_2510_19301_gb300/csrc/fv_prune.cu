@@ -22,11 +22,12 @@
 // weights with log-softmax normal emissions a step takes about 34 of 256 rows,
 // 40 of 512, 61 of 1000.
 //
-// Measured (GB300): 1024 sequences of 500 .. 4000 steps, K = 256: 17.4 -> 7.7
+// Measured (GB300): 1024 sequences of 500 .. 4000 steps, K = 256: 17.3 -> 7.6
 // ms per decode against the slot engine of fv_dense.cu; 150 sequences of 200
-// .. 1500 steps, K = 1000: 21.8 -> 7.3 ms; 8 sequences of 1500 steps, K = 4096:
-// 31.7 -> 17.3 ms; one K = 512 sequence of 512 steps: 1.81 -> 1.34 ms.  Bound now: latency and shared-memory wavefronts (at K =
-// 256, 650 wavefronts and 2200 warp instructions per job step), not the max.
+// .. 1500 steps, K = 1000: 21.8 -> 7.0 ms; 8 sequences of 1500 steps, K = 4096:
+// 31.7 -> 17.6 ms; one K = 512 sequence of 512 steps: 1.80 -> 1.37 ms.  Bound
+// now: latency and shared-memory wavefronts (at K = 256, 730 wavefronts and
+// 2270 warp instructions per job step), not the max.
 #include <cuda_runtime.h>
 #include <float.h>
 #include <math_constants.h>
