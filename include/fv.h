@@ -91,7 +91,9 @@ typedef enum { FV_EMIT_DENSE = 0, FV_EMIT_DISCRETE = 1 } fv_emit_kind;
  * serving loop): take the kernel configuration with the least SM time per
  * step rather than the one that finishes this call soonest on an idle GPU.
  * Today this keeps dense beams (P = 0) on one CTA per sequence, which takes
- * about a third of the SM time per step of one 8-CTA cluster per sequence.
+ * about a third of the SM time per step of one 8-CTA cluster per sequence,
+ * and at K > 1024 lets exact decoding hand no sequence to the engine that
+ * waits for the whole GPU.
  * Results are the same either way. */
 #define FV_SHARED_GPU 0x20u
 /* Test hook for failure detection: the first CTA of the whole-GPU engine
